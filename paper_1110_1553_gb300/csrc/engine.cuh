@@ -1496,6 +1496,7 @@ __device__ __forceinline__ void tc_setup(tc::State &ts) {
         ptx::mbar_init(&ts.img[c], 1);
       }
       ptx::mbar_init(&ts.done, 1);
+      for (int c = 0; c < tc::NB; ++c) ptx::mbar_init(&ts.ready[c], 1);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (threadIdx.x < 32) tc::tmem_alloc(&ts.tmem);
@@ -1519,8 +1520,8 @@ __device__ bool tc_task(const EngineParams &p, const Geo<Real> &g, const Task &t
   if constexpr (TC && sizeof(Real) == 4) {
     if (t.op == OP_GEQRT || t.op == OP_TSQRT || t.op == OP_TTQRT) {
       const int mode = t.op == OP_GEQRT ? 1 : (t.op == OP_TSQRT ? 0 : 2);
-      tc::panel(mode, g.tile(t.i, t.k), g.tile(t.r, t.k), g.tfac(mode == 1 ? 0 : 1, t.i, t.k), g.t32 != 0, dyn);
-      return true;
+      return tc::panel(mode, g.tile(t.i, t.k), g.tile(t.r, t.k), g.tfac(mode == 1 ? 0 : 1, t.i, t.k), g.t32 != 0, dyn,
+                       ts, tph, &sh.abort, p.timeout_ns);
     }
     const int mode = t.op == OP_UNMQR ? 1 : (t.op == OP_TSMQR ? 0 : 2);
     const bool pair = t.op != OP_UNMQR;

@@ -214,3 +214,24 @@ def test_split_launch_equals_one_launch():
     for (A, b), x in zip(host, outs[1]):
         xo = lstsq_unblocked(A.astype(np.float64), b)
         assert np.linalg.norm(x.cpu().numpy() - xo) / np.linalg.norm(xo) <= 1e-12
+
+
+@pytest.mark.parametrize("shape,a", [((1, 1), 1), ((2, 1), 2), ((2, 1), 1)])
+def test_panel_scaled_columns_tc(shape, a):
+    """GEQRT, TSQRT and TTQRT on columns scaled by powers of two whose squares
+    under- and overflow FP32 (the panel's scaled norms) and by 1 in between:
+    QR commutes with a column scaling, so R must be the unscaled R with scaled
+    columns, each column within the 5e-6 of the R tolerance of its own norm;
+    a zero column gives a zero column of R."""
+    m = shape[0]
+    A = inputs.gaussian(m * NB, NB, seed=760 + m + a).astype(np.float32)
+    recs = hqr_elim_list(m, 1, a, 1, FLAT, FLAT)
+    scale = np.ldexp(1.0, np.resize([0, -60, 60, 0, -90], NB)).astype(np.float32)
+    scale[[5, 77]] = 0.0
+    base = tile_qr((A * (scale != 0)).astype(np.float64), NB, NB, recs).R()
+    R = hqr.geqrf(torch.from_numpy(A * scale).cuda(), NB, NB, recs, tensor=True).R().cpu().numpy().astype(np.float64)
+    norms = np.linalg.norm(A.astype(np.float64), axis=0)
+    s = scale.astype(np.float64)
+    assert np.all(R[:, s == 0] == 0)
+    err = np.abs(R / np.where(s == 0, 1, s) - np.where(s == 0, 0, base))
+    assert np.max(err / norms) <= 5e-6
