@@ -14,13 +14,12 @@
 //
 // Arithmetic (compact-WY Householder, reflectors grouped ib at a time):
 //   column j of (alpha, x2): s = ||x2|| (sum of squares; a max-scaled second
-//   pass when the sum under- or overflows), beta = -sign(alpha) hypot(alpha,
-//   s) with sign(+-0) = +1, tau = (beta - alpha) / beta, v = (1, x2/(alpha -
+//   pass when the sum leaves a range around 1), beta = -sign(alpha) ||(alpha,
+//   s)|| with sign(+-0) = +1, tau = (beta - alpha) / beta, v = (1, x2/(alpha -
 //   beta)); s == 0 gives the identity (tau = 0, beta = alpha).
 //   T of a block: T[j,j] = tau_j, T[:j,j] = -tau_j T[:j,:j] (V[:,:j]^T v_j).
 //   Q^T C = C - V T^T V^T C (blocks in ascending order); Q C uses T and the
 //   descending order.
-// Norm reductions use warp shuffles and a per-warp shared-memory stage.
 #pragma once
 
 #include <algorithm>
@@ -37,16 +36,6 @@ constexpr int NT = 256;         // threads per CTA
 constexpr int NWARP = NT / 32;  // warps per CTA
 constexpr int IBMAX = 32;       // largest inner block
 
-template <typename Real>
-struct RealTraits;
-template <>
-struct RealTraits<double> {
-  static constexpr double tiny = 1e-280, huge = 1e280;  // sum-of-squares range kept unscaled
-};
-template <>
-struct RealTraits<float> {
-  static constexpr float tiny = 1e-30f, huge = 1e30f;
-};
 // shared-memory column padding (elements): keeps every staged column on a
 // 16-byte boundary and spreads columns over banks
 template <typename Real>
@@ -139,10 +128,10 @@ struct Shared {
   int norelease;     // the task released none of its successors (a gate that cancelled its rounds)
   int kept;          // a successor the last task made ready and this CTA runs next (-1: none)
   int popped;        // the task warp 1 claimed (-1: none, or finished)
-  Real red[2 * NWARP];
   Real tau[IBMAX];
-  Real wv[IBMAX];
-  Real bc[4];
+  Real sc[IBMAX];  // panel blocks: v_j = sc[j] x_j
+  Real snext;      // product of the current column with the next one
+  int redo;        // j + 1: column j was scaled in place, products formed before are void
 };
 
 // ---------------------------------------------------------------- helpers --
@@ -233,43 +222,6 @@ __device__ __forceinline__ Real warp_sum(Real v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
-}
-
-// Sum over the CTA; every thread gets the same value (fixed order). Only
-// threads below `nact` hold nonzero values, so warps beyond them skip their
-// reduction, and one thread adds the warps' partial sums and broadcasts the
-// total: in FP64 a warp-wide add occupies the SM's FP64 pipe for 16 cycles
-// whether or not its lanes need the result.
-template <typename Real>
-__device__ Real block_sum(Real v, Shared<Real> &sh, int nact = NT) {
-  if ((int)(threadIdx.x & ~31u) < nact) v = warp_sum(v);
-  if ((threadIdx.x & 31) == 0) sh.red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    Real t = 0;
-#pragma unroll
-    for (int q = 0; q < NWARP; ++q) t += sh.red[q];
-    sh.red[NWARP] = t;
-  }
-  __syncthreads();
-  return sh.red[NWARP];
-}
-
-template <typename Real>
-__device__ Real block_max(Real v, Shared<Real> &sh, int nact = NT) {
-  if ((int)(threadIdx.x & ~31u) < nact)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if ((threadIdx.x & 31) == 0) sh.red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    Real t = 0;
-#pragma unroll
-    for (int q = 0; q < NWARP; ++q) t = fmax(t, sh.red[q]);
-    sh.red[NWARP] = t;
-  }
-  __syncthreads();
-  return sh.red[NWARP];
 }
 
 // FP32 versions of the two GEMM phases with register blocking and 16-byte
@@ -533,125 +485,267 @@ __device__ void sub_top(Real *Ct, int ldt, const Real *W, int ldw, int Mi, int N
 
 enum { PANEL_GE = 0, PANEL_TS = 1, PANEL_TT = 2 };
 
-// Householder factorization of one block of ib columns held in shared memory.
-//  GE: P is L x ib, column jj has alpha = P(jj,jj) and x2 = P(jj+1:L, jj).
-//  TS: alpha = Rt(jj,jj), x2 = P(0:L, jj) (the killed square tile).
-//  TT: alpha = Rt(jj,jj), x2 = P(0:q0+jj+1, jj) (upper-triangular tile).
-// On return P holds the reflectors' lower parts (GE: R above) and sh.tau the
-// scalars; Rt's upper triangle holds the updated R rows of the block.
+// Scalars of the reflector that maps (alpha, x), ss = x^T x, to beta e_1:
+// with h = ||(alpha, x)||, beta = -sign(alpha) h, tau = (beta - alpha) / beta =
+// 1 + |alpha| / h, scale = 1 / (alpha - beta); alpha and ss in a range where
+// nothing under- or overflows. FP64 instructions of one warp issue 64 cycles
+// apart on this GPU, so the chain counts them: from the hardware's 20-bit
+// approximations of n2^(-1/2) and 1 / d, two terms of the binomial series of
+// (1 - e)^(-1/2) and of the geometric series of (1 - e)^(-1), e the residual
+// of the approximation by FMA, leave an error of order e^3 (below 2^-58):
+// 10 instructions, where a square root and two divisions take about 30.
+__device__ __forceinline__ void reflector_scalars(double alpha, double ss, double &beta, double &t, double &scale) {
+  const double n2 = fma(alpha, alpha, ss), aa = fabs(alpha);
+  double y0, z0;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(n2));
+  const double p = n2 * y0;
+  const double e = fma(-p, y0, 1.0);
+  const double q = e * fma(0.375, e, 0.5);
+  const double h = fma(p, q, p);
+  const double d = aa + h;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(z0) : "d"(d));
+  const double r = fma(-d, z0, 1.0);
+  const double z = fma(z0, fma(r, r, r), z0);
+  t = fma(aa, fma(y0, q, y0), 1.0);
+  // alpha >= 0 (either zero counts as positive), on its words
+  const int ah = __double2hiint(alpha);
+  const int flip = ah < 0 && ((ah << 1) | __double2loint(alpha)) != 0 ? (int)0x80000000 : 0;
+  beta = __hiloint2double(__double2hiint(h) ^ flip ^ (int)0x80000000, __double2loint(h));
+  scale = __hiloint2double(__double2hiint(z) ^ flip, __double2loint(z));
+}
+__device__ __forceinline__ void reflector_scalars(float alpha, float ss, float &beta, float &t, float &scale) {
+  tc::reflector_plain(alpha, ss, beta, t, scale);
+}
+
+// Sum over the warp of nonnegative values: FP32 by shuffles; FP64 in fixed
+// point, 59 bits below the largest value's exponent (each value cut by less
+// than 2^-58 of the largest) in three integer warp reductions, about half the
+// time of five shuffled FP64 additions. 0 where the exponent is extreme (or a
+// value not finite), which no caller takes for a plain sum.
+__device__ __forceinline__ float warp_sum_pos(float v) { return warp_sum(v); }
+__device__ __forceinline__ double warp_sum_pos(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v);
+  const unsigned E = __reduce_max_sync(0xffffffffu, hi) >> 20;
+  const unsigned e = hi >> 20, sh = E - e;
+  unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)__double2loint(v);
+  m = e == 0 || sh > 63 ? 0ull : (m << 6) >> sh;
+  const unsigned s0 = __reduce_add_sync(0xffffffffu, (unsigned)m & 0x3fffffu);
+  const unsigned s1 = __reduce_add_sync(0xffffffffu, (unsigned)(m >> 22) & 0x3fffffu);
+  const unsigned s2 = __reduce_add_sync(0xffffffffu, (unsigned)(m >> 44));
+  const double s = __ull2double_rn((unsigned long long)s0 + ((unsigned long long)s1 << 22) + ((unsigned long long)s2 << 44));
+  if (E < 200 || E > 1846) return 0.0;
+  return __hiloint2double(__double2hiint(s) + (((int)E - 1023 - 58) << 20), __double2loint(s));
+}
+
+// First and past-last row of column j of a block below its diagonal (GE) or
+// of the killed tile (TS: all, TT: the upper triangle).
+__device__ __forceinline__ int refl_begin(int mode, int j) { return mode == PANEL_GE ? j + 1 : 0; }
+__device__ __forceinline__ int refl_end(int mode, int j, int L, int q0) {
+  return mode == PANEL_TT ? min(L, q0 + j + 1) : L;
+}
+
+// sum of x[k] y[k], and y[k] += a x[k], over k = k, k + step, ... < k1. In FP32
+// four terms are loaded before the first is used (a store to y would otherwise
+// keep the next loads behind it); in FP64 the FMAs' issue interval covers the
+// loads, and the shorter code is faster.
 template <typename Real>
-__device__ void factor_block(int mode, Real *P, int ld, int L, int ib, Real *Rt, int ldt, int q0,
-                             Shared<Real> &sh) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int jj = 0; jj < ib; ++jj) {
-    const int r0 = (mode == PANEL_GE) ? jj + 1 : 0;
-    const int r1 = (mode == PANEL_TT) ? min(L, q0 + jj + 1) : L;
-    Real *col = P + (size_t)jj * ld;
-    const int nact = min(NT, r1 - r0);  // threads holding rows of the column
-    Real ss = 0;
-    for (int k = r0 + tid; k < r1; k += NT) ss = fma(col[k], col[k], ss);
-    ss = block_sum(ss, sh, nact);
-    Real snorm;
-    const bool plain = ss > RealTraits<Real>::tiny && ss < RealTraits<Real>::huge;
-    if constexpr (sizeof(Real) == 8) {
-      // FP64: the norm only matters to thread 0 below, which forms ||(alpha, x)|| from ss itself
-      // (a warp-wide square root on every warp would occupy the FP64 pipe for nothing)
-      snorm = plain ? ss : Real(0);
-    }
-    if (plain) {
-      if constexpr (sizeof(Real) == 4) snorm = sqrt(ss);
-    } else {
-      Real am = 0;
-      for (int k = r0 + tid; k < r1; k += NT) am = fmax(am, fabs(col[k]));
-      am = block_max(am, sh, nact);
-      if (am == Real(0)) {
-        snorm = 0;
-      } else {
-        const Real inv = Real(1) / am;
-        Real s2 = 0;
-        for (int k = r0 + tid; k < r1; k += NT) {
-          const Real x = col[k] * inv;
-          s2 = fma(x, x, s2);
-        }
-        s2 = block_sum(s2, sh, nact);
-        snorm = am * sqrt(s2);
+__device__ __forceinline__ Real strided_dot(const Real *x, const Real *y, int k, int k1, int step) {
+  Real a = 0;
+#pragma unroll 4
+  for (; k < k1; k += step) a = fma(x[k], y[k], a);
+  return a;
+}
+template <typename Real>
+__device__ __forceinline__ void strided_axpy(Real *y, const Real *x, Real a, int k, int k1, int step) {
+  if constexpr (sizeof(Real) == 4) {
+    for (; k + 3 * step < k1; k += 4 * step) {
+      Real xv[4], yv[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        xv[u] = x[k + u * step];
+        yv[u] = y[k + u * step];
       }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) y[k + u * step] = fma(a, xv[u], yv[u]);
     }
-    Real *diag = (mode == PANEL_GE) ? &col[jj] : &Rt[jj + (size_t)jj * ldt];
-    if (tid == 0) {
-      const Real alpha = *diag;
-      Real beta = alpha, t = 0, scale = 0;
-      if (snorm != Real(0)) {
-        Real h;
-        if constexpr (sizeof(Real) == 8)  // unscaled: snorm holds ss; sqrt(alpha^2 + ss) cannot overflow
-          h = plain ? (fabs(alpha) < 1e150 ? sqrt(fma(alpha, alpha, ss)) : hypot(alpha, sqrt(ss)))
-                    : hypot(alpha, snorm);
-        else
-          h = hypot(alpha, snorm);
-        beta = (alpha >= Real(0)) ? -h : h;
-        t = (beta - alpha) / beta;
-        scale = Real(1) / (alpha - beta);
+  }
+#pragma unroll 2
+  for (; k < k1; k += step) y[k] = fma(a, x[k], y[k]);
+}
+
+// lo < ss < hi and |alpha| < hi, on the high words of FP64 values (an FP64
+// comparison issues like any other FP64 instruction; NaN is out of range).
+__device__ __forceinline__ bool in_plain_range(double alpha, double ss) {
+  constexpr int lo = 0x37a00000, hi = 0x48400000;  // 2^-133, 2^133: about 1e-40 and 1e40
+  return __double2hiint(ss) > lo && __double2hiint(ss) < hi && (__double2hiint(alpha) & 0x7fffffff) < hi;
+}
+__device__ __forceinline__ bool in_plain_range(float alpha, float ss) {
+  return ss > 1e-12f && ss < 1e12f && fabsf(alpha) < 1e12f;
+}
+
+// Norm and scalars of column j by one warp (ss: this lane's share of its sum
+// of squares). Columns in the plain range stay as they are and are scaled at
+// the end of the block (v = sh.sc[j] x); others are scaled here in place
+// (sh.sc[j] = 1, sh.redo = j + 1: the products already formed with the column
+// are void).
+template <typename Real>
+__device__ __forceinline__ void form_reflector(int mode, Real *P, int ld, int L, Real *Rt, int ldt, int q0, int j, Real ss,
+                                               Shared<Real> &sh) {
+  const int lane = threadIdx.x & 31;
+  Real *col = P + (size_t)j * ld;
+  Real *diag = mode == PANEL_GE ? col + j : Rt + j + (size_t)j * ldt;
+  const Real alpha = *diag;
+  const Real sum = warp_sum_pos(ss);
+  Real beta = alpha, t = 0, scale = 0;
+  if (in_plain_range(alpha, sum)) {
+    reflector_scalars(alpha, sum, beta, t, scale);
+  } else {
+    const int r0 = refl_begin(mode, j), r1 = refl_end(mode, j, L, q0);
+    Real am = 0;
+    for (int k = r0 + lane; k < r1; k += 32) am = fmax(am, fabs(col[k]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) am = fmax(am, __shfl_xor_sync(0xffffffffu, am, o));
+    if (am != Real(0)) {
+      const Real inv = Real(1) / am;
+      Real s2 = 0;
+      for (int k = r0 + lane; k < r1; k += 32) {
+        const Real x = col[k] * inv;
+        s2 = fma(x, x, s2);
       }
-      *diag = beta;
-      sh.tau[jj] = t;
-      sh.bc[0] = t;
-      sh.bc[1] = scale;
+      const Real h = hypot(alpha, am * sqrt(warp_sum(s2)));
+      beta = alpha >= Real(0) ? -h : h;
+      t = (beta - alpha) / beta;
+      const Real sc = Real(1) / (alpha - beta);
+      for (int k = r0 + lane; k < r1; k += 32) col[k] *= sc;
+      scale = 1;
+      if (lane == 0) sh.redo = j + 1;
     }
-    __syncthreads();
-    const Real t = sh.bc[0], scale = sh.bc[1];
-    for (int k = r0 + tid; k < r1; k += NT) col[k] *= scale;
-    __syncthreads();
-    if (t == Real(0)) continue;  // identity reflector: nothing to apply
-    // w_c = top(jj,c) + v^T P(:,c) for the block's later columns; short columns share a warp
-    // (LPC lanes per column, 32 / LPC columns per warp), which saves shuffle-add levels
-    const int nr = r1 - r0, ncl = ib - jj - 1;
-    const int LPC = nr > 64 ? 32 : (nr > 32 ? 16 : 8), CPW = 32 / LPC;
-    const int sub = lane / LPC, sl = lane - sub * LPC;
-    for (int cw0 = jj + 1 + warp * CPW; cw0 < ib; cw0 += NWARP * CPW) {
-      const int c = cw0 + sub;
-      const bool on = c < ib;
-      const Real *pc = P + (size_t)(on ? c : jj) * ld;
-      Real s = 0;
-      if (on)
-        for (int k = r0 + sl; k < r1; k += LPC) s = fma(col[k], pc[k], s);
-      for (int o = LPC >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (on && sl == 0) {
-        const Real top = (mode == PANEL_GE) ? pc[jj] : Rt[jj + (size_t)c * ldt];
-        sh.wv[c] = t * (top + s);
-      }
-    }
-    __syncthreads();
-    for (int e = tid; e < nr * ncl; e += NT) {
-      const int c = jj + 1 + e / nr, k = r0 + e % nr;
-      Real *pc = P + (size_t)c * ld;
-      pc[k] = fma(-col[k], sh.wv[c], pc[k]);
-    }
-    if (tid > jj && tid < ib) {
-      if (mode == PANEL_GE)
-        P[jj + (size_t)tid * ld] -= sh.wv[tid];
-      else
-        Rt[jj + (size_t)tid * ldt] -= sh.wv[tid];
-    }
-    __syncthreads();
+  }
+  __syncwarp();
+  if (lane == 0) {
+    *diag = beta;
+    sh.tau[j] = t;
+    sh.sc[j] = scale;
   }
 }
 
-// T of a block from the Gram matrix G = V^T V (only G(l, j), l < j, used).
+// Householder factorization of one block of ib columns held in shared memory,
+// and the block's T.
+//  GE: P is L x ib, column jj has alpha = P(jj,jj) and x2 = P(jj+1:L, jj).
+//  TS: alpha = Rt(jj,jj), x2 = P(0:L, jj) (the killed square tile).
+//  TT: alpha = Rt(jj,jj), x2 = P(0:q0+jj+1, jj) (upper-triangular tile).
+// On return P holds the reflectors' lower parts (GE: R above), Rt's upper
+// triangle the updated R rows of the block, and Tq (leading dimension ldq) its
+// upper-triangular T. G: scratch of ib x ib.
+//
+// Eight lanes hold a column. Step j: warp 0 applies reflector j - 1 to column
+// j with all its lanes and forms reflector j, while the column groups apply
+// reflector j - 1 to the columns after j and form the products of column j, as
+// it is, with every other column: w_c = tau (top + scale x^T a_c) when the
+// scalars arrive, or the Gram entry G(c, j) of an earlier column, from which
+// warp 1 forms T(:, j - 2). So a step costs one norm and its scalars, not the
+// sum of norm, scaling, products and updates with a barrier after each. In
+// FP64 it is bound by the chain of warp 0's instructions (64 cycles each), and
+// for blocks of 32 columns by the FP64 pipe; in FP32 by latencies. Cycles per
+// column (TS, one CTA): 64 x 16 FP64 3200, 256 x 32 FP64 11200, 128 x 16 FP32
+// 1700; block tasks of the whole engine: 64 x 16 FP64 68 -> 29 us, 128 x 32
+// 273 -> 155 us against one CTA-wide reduction after the other.
 template <typename Real>
-__device__ void build_t(Real *Tq, int ldq, const Real *G, int ib, const Shared<Real> &sh) {
-  for (int e = threadIdx.x; e < ib * ldq; e += NT) Tq[e] = 0;
-  __syncthreads();
-  for (int jj = 0; jj < ib; ++jj) {
-    const int tid = threadIdx.x;
-    if (tid < jj) {
-      Real y = 0;
-      for (int l = tid; l < jj; ++l) y = fma(Tq[tid + (size_t)l * ldq], G[l + (size_t)jj * ib], y);
-      Tq[tid + (size_t)jj * ldq] = -sh.tau[jj] * y;
-    } else if (tid == jj) {
-      Tq[jj + (size_t)jj * ldq] = sh.tau[jj];
+__device__ void factor_block(int mode, Real *P, int ld, int L, int ib, Real *Rt, int ldt, int q0, Real *Tq, int ldq,
+                             Real *G, Shared<Real> &sh) {
+  constexpr int LPC = 8, CPW = 32 / LPC;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int first = NWARP - (ib + CPW - 1) / CPW;  // column warps: first .. NWARP - 1
+  const int grp = warp - first;
+  const int part = lane & (LPC - 1), c = grp * CPW + lane / LPC;
+  const bool colw = grp >= 0 && grp * CPW < ib, has = colw && c < ib;
+  Real *pc = P + (size_t)(has ? c : 0) * ld;
+  Real s = 0;  // x_j^T a_c (every lane of the column's group)
+  auto products = [&](int j) {  // column j with this group's column
+    const Real *col = P + (size_t)j * ld;
+    const int r1 = refl_end(mode, j, L, q0);
+    __syncwarp();  // this group's column, updated by other lanes of it
+    Real a = strided_dot(col, pc, refl_begin(mode, j) + part, r1, LPC);
+#pragma unroll
+    for (int o = LPC >> 1; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    s = a;
+    if (c == j + 1 && has && part == 0) sh.snext = s;
+  };
+  auto apply = [&](int i, int from) {  // reflector i to columns >= from; G(c, i) of columns < i
+    const Real tau = sh.tau[i], sc = sh.sc[i];
+    const bool later = has && c >= from, earlier = has && c < i;
+    Real *top = mode == PANEL_GE || earlier ? pc + i : Rt + i + (size_t)(has ? c : 0) * ldt;
+    const Real base = mode == PANEL_GE || later ? *top : Real(0);
+    const Real w = (later ? tau : sh.sc[has ? c : 0]) * fma(sc, s, base);
+    __syncwarp();
+    if (later) {
+      strided_axpy(pc, P + (size_t)i * ld, -(sc * w), refl_begin(mode, i) + part, refl_end(mode, i, L, q0), LPC);
+      if (part == 0) *top = base - w;
+    } else if (earlier && part == 0) {
+      G[c + (size_t)i * ib] = w;
     }
+  };
+  auto t_column = [&](int j) {  // T(:, j) = -tau_j T(:, :j) G(:j, j), one row per lane
+    if (lane >= ib) return;
+    Real y = 0;
+#pragma unroll 4
+    for (int l = 0; l < j; ++l) y = fma(Tq[lane + (size_t)l * ldq], G[l + (size_t)j * ib], y);
+    const Real tau = sh.tau[j];
+    Tq[lane + (size_t)j * ldq] = lane < j ? -tau * y : (lane == j ? tau : Real(0));
+  };
+  if (tid == 0) sh.redo = 0;
+  __syncthreads();
+  for (int j = 0; j < ib; ++j) {
+    Real *cj = P + (size_t)j * ld;
+    if (warp == 0) {
+      Real ss = 0;
+      const int r1 = refl_end(mode, j, L, q0);
+      if (j > 0) {
+        const int i = j - 1;
+        const Real *col = P + (size_t)i * ld;
+        Real *top = mode == PANEL_GE ? cj + i : Rt + i + (size_t)j * ldt;
+        const Real base = *top, sc = sh.sc[i], w = sh.tau[i] * fma(sc, sh.snext, base), nw = -(sc * w);
+        // TT: row q0 + j of column i is zero
+#pragma unroll 2
+        for (int k = refl_begin(mode, i) + lane; k < r1; k += 32) {
+          const Real x = fma(nw, col[k], cj[k]);
+          cj[k] = x;
+          if (mode != PANEL_GE || k > j) ss = fma(x, x, ss);  // GE: row j is alpha
+        }
+        __syncwarp();
+        asm volatile("bar.arrive 1, %0;" ::"n"(NT) : "memory");
+        if (lane == 0) *top = base - w;
+      } else {
+        for (int k = refl_begin(mode, 0) + lane; k < r1; k += 32) ss = fma(cj[k], cj[k], ss);
+      }
+      form_reflector(mode, P, ld, L, Rt, ldt, q0, j, ss, sh);
+    }
+    if (colw && j > 0) apply(j - 1, j + 1);
+    if (warp != 0 && j > 0) asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
+    if (warp == 1 && j > 1) t_column(j - 2);
+    if (colw) products(j);
     __syncthreads();
+    if (sh.redo == j + 1) {  // the column was scaled in place (the same in every thread)
+      if (colw) products(j);
+      __syncthreads();
+    }
   }
+  if (colw) apply(ib - 1, ib);
+  __syncthreads();
+  if (warp == 1) {
+    if (ib > 1) t_column(ib - 2);
+    __syncwarp();
+    t_column(ib - 1);
+  } else {  // v = scale x
+    for (int cc = warp == 0 ? 0 : warp - 1; cc < ib; cc += NWARP - 1) {
+      const Real sc = sh.sc[cc];
+      if (sc == Real(1)) continue;
+      Real *col = P + (size_t)cc * ld;
+      const int r1 = refl_end(mode, cc, L, q0);
+      for (int k = refl_begin(mode, cc) + lane; k < r1; k += 32) col[k] *= sc;
+    }
+  }
+  __syncthreads();
 }
 
 // Set the structural zeros (and unit diagonal) of a staged V chunk.
@@ -793,7 +887,7 @@ __device__ void task_panel(const EngineParams &p, const Geo<Real> &g, const Task
       }
       __syncthreads();
     }
-    factor_block(mode, P, lds, L, ib, Rt, ldt, q0, sh);
+    factor_block(mode, P, lds, L, ib, Rt, ldt, q0, Tq, ldq, G, sh);
     // write back the factored block
     if (mode == PANEL_GE) {
       store_cols(XB + (size_t)q0 * nb + q0, nb, P, lds, L, ib, 0, 0);
@@ -802,9 +896,7 @@ __device__ void task_panel(const EngineParams &p, const Geo<Real> &g, const Task
       store_cols(XB + (size_t)q0 * nb, nb, P, lds, L, ib, mode == PANEL_TT ? 1 : 0, q0);
     }
     __syncthreads();
-    if (mode == PANEL_GE) shape_v(P, lds, L, ib, PANEL_GE, 0, 0);
-    gemm_tn(G, ib, P, lds, P, lds, L, ib, ib, (const Real *)nullptr, 0, scr);
-    build_t(Tq, ldq, G, ib, sh);
+    if (mode == PANEL_GE && t.blk == 0) shape_v(P, lds, L, ib, PANEL_GE, 0, 0);
     store_cols(Tg + (size_t)q * ib * ib, ib, Tq, ldq, ib, ib, 0, 0);
     if (t.blk > 0) break;
     // trailing columns of the tile(s): block reflector applied with Q^T

@@ -299,3 +299,30 @@ def test_split_panels_least_squares_plan():
     assert plan.status() == 0
     xo = lstsq_unblocked(A, b)
     assert np.linalg.norm(x.cpu().numpy() - xo) / np.linalg.norm(xo) <= 1e-12
+
+
+@pytest.mark.parametrize("shape,a,nb,ib", [((1, 1), 1, 64, 16), ((2, 1), 2, 64, 16), ((2, 1), 1, 64, 16), ((2, 1), 2, 24, 6),
+                                           ((2, 1), 1, 256, 32), ((2, 1), 2, 16, 16), ((2, 2), 2, 8, 2)])
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_panel_scaled_columns(shape, a, nb, ib, dtype):
+    """GEQRT, TSQRT and TTQRT blocks on columns whose sums of squares lie inside
+    and far outside the range whose columns are used unscaled: QR commutes
+    with a column scaling by powers of two, so R must be the unscaled R with
+    scaled columns, each column within R_TOL (FP32: 5e-6) of its own norm; zero
+    columns stay zero."""
+    if dtype == "f32" and ib % 4:
+        pytest.skip("FP32 inner blocks are multiples of 4")
+    m, n = shape
+    A = inputs.gaussian(m * nb, n * nb, seed=170 + nb + a)
+    recs = hqr_elim_list(m, n, a, 1, FLAT, FLAT)
+    exps = [0, -400, 400, 0, -60, 60, -480] if dtype == "f64" else [0, -60, 60, 0, -30, 30, -90]
+    scale = np.ldexp(1.0, np.resize(exps, n * nb))
+    scale[[1, 6]] = 0.0
+    A = A.astype(np.float32).astype(np.float64) if dtype == "f32" else A
+    base = tile_qr(A * (scale != 0), nb, ib, recs).R()
+    As = torch.from_numpy(A * scale).cuda()
+    R = hqr.geqrf(As if dtype == "f64" else As.float(), nb, ib, recs).R().double().cpu().numpy()
+    assert np.all(R[:, scale == 0] == 0)
+    keep = scale != 0
+    err = np.abs(R[:, keep] / scale[keep] - base[:, keep]) / np.linalg.norm(A, axis=0)[keep]
+    assert np.max(err) <= (R_TOL if dtype == "f64" else 5e-6)
