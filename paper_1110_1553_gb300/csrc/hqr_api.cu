@@ -273,11 +273,6 @@ int split_ib_for(int prec, const Problem &P) {
   return P.ib;
 }
 
-// Tuning of the column-slab widths for a tile size and precision. FP64 work
-// is bound by the FP64 pipe, so narrow slabs (more parallel tasks) cost
-// nothing; FP32 tasks are bound by their barriers and staging, so they take
-// wider slabs (more arithmetic per barrier) within the shared memory of two
-// CTAs per SM.
 bool prec_ok(int prec) { return prec == HQR_FP64 || prec == HQR_FP32 || prec == HQR_FP32_BF16X3; }
 
 // Tiles of this size on the tensor-core kernels (with one full T per tile).
@@ -300,7 +295,23 @@ void drop_t32(int prec, Problem &P) {
   P.tstr = (int)t_record(prec, P.nb, P.ib, false);
 }
 
-void choose_widths(int prec, int nb, int ib, Problem &P) {
+// Column-slab widths for a tile size and precision. A launch of few tiles is
+// bound by its chain of tasks, so its updates are cut narrow (shorter tasks on
+// more SMs); a launch of many tiles by the tasks' own cost, of which staging V
+// once per slab is a part, and so is the host's construction of the graph.
+// `tiles`: tiles of the factorization; 0 for plans and server requests, whose
+// launches hold other problems too and whose results must not depend on them
+// (the order of sums follows the width).
+// FP64 (ms, slabs of 16 / 8 / 4): 8 x 8 tiles of 64 2.66 / 2.52 / 2.40, 8 x 2
+// of 128 2.35 / 2.06 / 1.95, 16 x 16 of 64 6.1 / 5.7 / 6.0, 63 x 8 of 64 4.7 /
+// 5.3 / 8.0; inner blocks of 32 (more arithmetic per staged block): 16 x 16 of
+// 128 28.5 / 25.1 / 26.8, 32 x 16 of 128 47.8 / 42.7 / 57, 128 x 8 of 256
+// 259.5 / 255.5 (and 66 ms more on the host, so it stays at 16). FP32 on CUDA cores (slabs of 64 / 32 / 16): 20 x 14 of 128
+// 22.5 / 21.7 / 12.3 and 64 x 4 of 128 4.8 / 4.7 / 2.9 (slabs no wider than a
+// block also let the panels split, see split_ib_for), 10 x 5 of 64 1.29 / 1.25
+// / 1.10, 32 x 32 of 64 15.7 / 15.3 / 12.5 and of 128 47 / 46 / 29.5, 128 x 16 of
+// 128 29.8 / 29.2 / 35.7, 160 uneven problems 19.6 / 21.1 / 27.7.
+void choose_widths(int prec, int nb, int ib, Problem &P, long long tiles = 0) {
   P.wb = std::min(16, nb);
   P.tc = use_tc(prec, nb) ? 1 : 0;
   P.t32 = 1;
@@ -313,10 +324,13 @@ void choose_widths(int prec, int nb, int ib, Problem &P) {
   }
   if (prec == HQR_FP64) {
     P.w = std::min(16, nb);
+    if (tiles > 0 && nb >= 16) P.w = tiles <= 128 && ib <= 16 ? 4 : (tiles <= (nb >= 128 && ib > 16 ? 512 : 320) ? 8 : 16);
     P.wt = nb > 128 ? 8 : std::min(16, nb);
     P.vc = nb > 128 ? std::min(ib, 8) : std::min(ib, 16);
   } else {
     P.w = nb >= 256 ? 32 : std::min(64, nb);
+    // (fewer than 12 tiles keep whole panels)
+    if (tiles >= 12 && tiles <= 1024 && ib <= 16 && nb >= 16) P.w = 16;
     P.wt = nb >= 256 ? 16 : std::min(32, nb);
     P.vc = std::min(ib, 16);
   }
@@ -514,7 +528,7 @@ int hqr_task_graph(int m, int n, int nb, int ib, int prec, const hqr_elim_t *lis
   P.n = n;
   P.nb = nb;
   P.ib = ib;
-  choose_widths(prec, nb, ib, P);
+  choose_widths(prec, nb, ib, P, kind < 3 ? (long long)m * n : 0);
   const std::vector<PanelOp> ops = expand_ops(list, count, m, n);
   Graph g;
   if (kind == 0)
@@ -570,7 +584,7 @@ int hqr_geqrf(const void *dA, int M, int N, int lda, int prec, int nb, int ib, c
   F->prob.n = F->n;
   F->prob.nb = nb;
   F->prob.ib = ib;
-  choose_widths(prec, nb, ib, F->prob);
+  choose_widths(prec, nb, ib, F->prob, (long long)F->m * F->n);
   if (list) {
     if (hqr_validate_list(F->m, F->n, list, count) != HQR_SUCCESS) {
       delete F;
@@ -1797,7 +1811,7 @@ extern "C" int hqr_critical_path(int m, int n, int nb, int ib, int prec, const h
   pb.n = n;
   pb.nb = nb;
   pb.ib = ib;
-  choose_widths(prec, nb, ib, pb);
+  choose_widths(prec, nb, ib, pb, (long long)m * n);
   const Graph g = build_factor_graph(expand_ops(list, count, m, n), m, n, nb, pb.w, 0, split_ib_for(prec, pb));
   *critical_path = critical_path_length(g, nb);
   *work = total_cost(g, nb);
