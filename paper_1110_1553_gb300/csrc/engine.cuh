@@ -168,38 +168,71 @@ struct Copy {
   int nrows, ncols;
 };
 
-// Stage up to 3 column-blocks global -> shared with bulk copies, one copy per
-// column, and wait for them (bounded). Callers sync before (dst free).
+// Walks the elements r < n of columns c = 0, 1, ... in the order tid, tid + NT,
+// ... of the flattened index, with one division per walk.
+struct ColWalk {
+  int c, r, dc, dr, n;
+  __device__ explicit ColWalk(int rows) : n(rows) {
+    c = (int)threadIdx.x / n;
+    r = (int)threadIdx.x - c * n;
+    dc = NT / n;
+    dr = NT - dc * n;
+  }
+  __device__ void next() {
+    c += dc;
+    r += dr;
+    if (r >= n) {
+      r -= n;
+      ++c;
+    }
+  }
+};
+
+// Stage column-blocks global -> shared and wait for them. Columns of 2 KB and
+// more come by one bulk copy each (bounded wait); shorter ones by 16-byte
+// asynchronous copies of all threads (L2 only): a bulk copy takes about 60
+// cycles to issue whatever its size: the 288 columns of a 128 x 128 FP32 tile,
+// its T and C took 8 us, and take 2 us this way. Callers sync before (dst free).
+constexpr int kBulkBytes = 2048;
 template <typename Real>
 __device__ void stage(const EngineParams &p, Shared<Real> &sh, const Copy<Real> *cp, int ncp,
                       uint32_t &phase) {
   uint32_t total = 0;
-  for (int q = 0; q < ncp; ++q)
-    if (cp[q].nrows > 0 && cp[q].ncols > 0)
-      total += (uint32_t)cp[q].nrows * (uint32_t)sizeof(Real) * (uint32_t)cp[q].ncols;
-  if (total == 0) return;
-  if (threadIdx.x < 32) {
+  for (int q = 0; q < ncp; ++q) {
+    const uint32_t bytes = (uint32_t)cp[q].nrows * (uint32_t)sizeof(Real);
+    if (cp[q].nrows > 0 && bytes >= (uint32_t)kBulkBytes) total += bytes * (uint32_t)cp[q].ncols;
+  }
+  if (total > 0 && threadIdx.x < 32) {
     ptx::fence_proxy_async();
     if (threadIdx.x == 0) ptx::mbar_arrive_expect_tx(&sh.bar, total);
     __syncwarp();
     for (int q = 0; q < ncp; ++q) {
-      if (cp[q].nrows <= 0) continue;
       const uint32_t bytes = (uint32_t)cp[q].nrows * (uint32_t)sizeof(Real);
+      if (cp[q].nrows <= 0 || bytes < (uint32_t)kBulkBytes) continue;
       for (int c = threadIdx.x; c < cp[q].ncols; c += 32)
         ptx::bulk_g2s(cp[q].dst + (size_t)c * cp[q].ldd, cp[q].src + (long long)c * cp[q].lds, bytes,
                       &sh.bar);
     }
   }
-  if (!ptx::mbar_try_wait(&sh.bar, phase)) {
-    const uint64_t t0 = ptx::globaltimer();
-    while (!ptx::mbar_try_wait(&sh.bar, phase)) {
-      if (sh.abort || ptx::globaltimer() - t0 > (uint64_t)p.timeout_ns) {
-        sh.abort = 1;
-        break;
+  constexpr int E = 16 / (int)sizeof(Real);  // elements per 16 bytes
+  for (int q = 0; q < ncp; ++q) {
+    if (cp[q].nrows <= 0 || cp[q].nrows * (int)sizeof(Real) >= kBulkBytes) continue;
+    for (ColWalk w(cp[q].nrows / E); w.c < cp[q].ncols; w.next())
+      ptx::cp_async16(cp[q].dst + (size_t)w.c * cp[q].ldd + w.r * E, cp[q].src + (long long)w.c * cp[q].lds + w.r * E);
+  }
+  ptx::cp_async_wait_all();
+  if (total > 0) {
+    if (!ptx::mbar_try_wait(&sh.bar, phase)) {
+      const uint64_t t0 = ptx::globaltimer();
+      while (!ptx::mbar_try_wait(&sh.bar, phase)) {
+        if (sh.abort || ptx::globaltimer() - t0 > (uint64_t)p.timeout_ns) {
+          sh.abort = 1;
+          break;
+        }
       }
     }
+    phase ^= 1u;
   }
-  phase ^= 1u;
   __syncthreads();
   if (sh.abort && threadIdx.x == 0) set_error(p, HQR_ERR_TIMEOUT, -1);
 }
@@ -209,11 +242,9 @@ __device__ void stage(const EngineParams &p, Shared<Real> &sh, const Copy<Real> 
 template <typename Real>
 __device__ void store_cols(Real *g, long long ldg, const Real *s, int ldsm, int nrows, int ncols, int mode,
                            int roff) {
-  const int total = nrows * ncols;
-  for (int e = threadIdx.x; e < total; e += NT) {
-    const int c = e / nrows, r = e - c * nrows;
-    if (mode == 1 && r > roff + c) continue;
-    g[(long long)c * ldg + r] = s[(size_t)c * ldsm + r];
+  for (ColWalk w(nrows); w.c < ncols; w.next()) {
+    if (mode == 1 && w.r > roff + w.c) continue;
+    g[(long long)w.c * ldg + w.r] = s[(size_t)w.c * ldsm + w.r];
   }
 }
 
@@ -232,7 +263,7 @@ __device__ __forceinline__ Real warp_sum(Real v) {
 __device__ void gemm_tn_f32(float *W, int ldw, const float *V, int ldv, const float *Cm, int ldc, int K, int Mi,
                             int Nj, const float *Cinit, int ldi, float *scr) {
   const int ti = (Mi + 3) >> 2, tj = (Nj + 3) >> 2, T = ti * tj;
-  int G = NT / T;
+  int G = NT / T;  // groups of the K range
   if (G < 1) G = 1;
   if (G > 4) G = 4;
   int Kc = (K + G - 1) / G;
@@ -267,36 +298,39 @@ __device__ void gemm_tn_f32(float *W, int ldw, const float *V, int ldv, const fl
           acc[a][b] = fmaf(v4[a].w, c4[b].w, acc[a][b]);
         }
     }
-    float *dst = scr + (size_t)(g * T + mt) * 16;
+    // row a of the block at ((a * T G) + unit) * 4: consecutive threads, consecutive 16 bytes
+    float4 *dst = reinterpret_cast<float4 *>(scr) + u;
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) dst[a * 4 + b] = acc[a][b];
+    for (int a = 0; a < 4; ++a) dst[a * T * G] = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
   }
   __syncthreads();
   for (int o = threadIdx.x; o < Mi * Nj; o += NT) {
     const int i = o % Mi, j = o / Mi;
-    const int mt = (i >> 2) + (j >> 2) * ti, q = (i & 3) * 4 + (j & 3);
+    const int mt = (i >> 2) + (j >> 2) * ti;
+    const float *q = scr + ((size_t)(i & 3) * T * G + mt) * 4 + (j & 3);
     float s = 0.f;
-    for (int g = 0; g < G; ++g) s += scr[(size_t)(g * T + mt) * 16 + q];
+#pragma unroll 4
+    for (int g = 0; g < G; ++g) s += q[(size_t)g * T * 4];
     W[i + (size_t)j * ldw] = (Cinit ? Cinit[i + (size_t)j * ldi] : 0.f) + s;
   }
   __syncthreads();
 }
 
-__device__ void gemm_nn_sub_f32(float *Cm, int ldc, const float *V, int ldv, const float *W, int ldw, int K, int Mi,
-                                int Nj) {
-  const int tk = K >> 2, tj = (Nj + 7) >> 3;
+template <int CH>
+__device__ __forceinline__ void gemm_nn_sub_f32(float *Cm, int ldc, const float *V, int ldv, const float *W, int ldw,
+                                                int K, int Mi, int Nj) {
+  const int tk = K >> 2, tj = (Nj + CH - 1) / CH;
   for (int u = threadIdx.x; u < tk * tj; u += NT) {
-    const int k0 = (u % tk) * 4, j0 = (u / tk) * 8, jn = min(8, Nj - j0);
-    float4 acc[8];
+    const int k0 = (u % tk) * 4, j0 = (u / tk) * CH, jn = min(CH, Nj - j0);
+    float4 acc[CH];
 #pragma unroll
-    for (int b = 0; b < 8; ++b) acc[b] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int b = 0; b < CH; ++b) acc[b] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll CH == 2 ? 4 : 1
     for (int i = 0; i < Mi; ++i) {
       const float4 v = *reinterpret_cast<const float4 *>(V + (size_t)i * ldv + k0);
       const float *w = W + i + (size_t)j0 * ldw;
 #pragma unroll
-      for (int b = 0; b < 8; ++b) {
+      for (int b = 0; b < CH; ++b) {
         const float wb = b < jn ? w[(size_t)b * ldw] : 0.f;
         acc[b].x = fmaf(v.x, wb, acc[b].x);
         acc[b].y = fmaf(v.y, wb, acc[b].y);
@@ -305,7 +339,7 @@ __device__ void gemm_nn_sub_f32(float *Cm, int ldc, const float *V, int ldv, con
       }
     }
 #pragma unroll
-    for (int b = 0; b < 8; ++b)
+    for (int b = 0; b < CH; ++b)
       if (b < jn) {
         float4 *c = reinterpret_cast<float4 *>(Cm + (size_t)(j0 + b) * ldc + k0);
         float4 x = *c;
@@ -321,7 +355,8 @@ __device__ void gemm_nn_sub_f32(float *Cm, int ldc, const float *V, int ldv, con
 
 // W(i,j) = [Cinit(i,j)] + sum_{k<K} V(k,i) C(k,j), i < Mi, j < Nj.
 // Short output sets split K among thread groups; partial sums are combined
-// in a fixed order through `scr` (>= NT elements).
+// in a fixed order through `scr` (>= NT elements; FP32: 16 per output block of
+// 4 x 4 and thread group, at most 4 groups).
 template <typename Real>
 __device__ void gemm_tn(Real *W, int ldw, const Real *V, int ldv, const Real *Cm, int ldc, int K, int Mi,
                         int Nj, const Real *Cinit, int ldi, Real *scr) {
@@ -378,33 +413,46 @@ __device__ void gemm_tn(Real *W, int ldw, const Real *V, int ldv, const Real *Cm
 // The FP64 version accumulates into C itself (C = fma(-V, W, C), terms in
 // ascending i): a separate subtraction per output would cost the FP64 pipe
 // as much as a DFMA, one extra operation per Mi (as few as 8) DFMAs.
+// A thread takes CH columns of a row (FP32: of four rows): 8, or fewer where
+// that would leave quarters of the SM without a warp.
+template <int CH>
+__device__ __forceinline__ void gemm_nn_sub_f64(double *Cm, int ldc, const double *V, int ldv, const double *W, int ldw,
+                                                int K, int Mi, int Nj) {
+  const int total = K * ((Nj + CH - 1) / CH);
+  for (int it = threadIdx.x; it < total; it += NT) {
+    const int k = it % K, j0 = (it / K) * CH, jn = min(CH, Nj - j0);
+    double acc[CH];
+#pragma unroll
+    for (int q = 0; q < CH; ++q) acc[q] = q < jn ? Cm[k + (size_t)(j0 + q) * ldc] : 0.0;
+    for (int i = 0; i < Mi; ++i) {
+      const double v = V[k + (size_t)i * ldv];
+      const double *w = W + i + (size_t)j0 * ldw;
+#pragma unroll
+      for (int q = 0; q < CH; ++q)
+        if (q < jn) acc[q] = fma(-v, w[(size_t)q * ldw], acc[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < CH; ++q)
+      if (q < jn) Cm[k + (size_t)(j0 + q) * ldc] = acc[q];
+  }
+  __syncthreads();
+}
+
 template <typename Real>
 __device__ void gemm_nn_sub(Real *Cm, int ldc, const Real *V, int ldv, const Real *W, int ldw, int K, int Mi,
                             int Nj) {
   if constexpr (sizeof(Real) == 4) {
-    gemm_nn_sub_f32(Cm, ldc, V, ldv, W, ldw, K, Mi, Nj);
-    return;
+    const int tk = K >> 2;
+    if (tk * ((Nj + 7) >> 3) >= NT || Nj > 16)
+      gemm_nn_sub_f32<8>(Cm, ldc, V, ldv, W, ldw, K, Mi, Nj);
+    else
+      gemm_nn_sub_f32<2>(Cm, ldc, V, ldv, W, ldw, K, Mi, Nj);
+  } else {
+    if (K * ((Nj + 7) >> 3) >= NT / 2)
+      gemm_nn_sub_f64<8>(Cm, ldc, V, ldv, W, ldw, K, Mi, Nj);
+    else
+      gemm_nn_sub_f64<2>(Cm, ldc, V, ldv, W, ldw, K, Mi, Nj);
   }
-  const int nchunk = (Nj + 7) / 8;
-  const int total = K * nchunk;
-  for (int it = threadIdx.x; it < total; it += NT) {
-    const int k = it % K, jc = it / K;
-    const int j0 = jc * 8, jn = min(8, Nj - j0);
-    Real acc[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = q < jn ? Cm[k + (size_t)(j0 + q) * ldc] : Real(0);
-    for (int i = 0; i < Mi; ++i) {
-      const Real v = V[k + (size_t)i * ldv];
-      const Real *w = W + i + (size_t)j0 * ldw;
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (q < jn) acc[q] = fma(-v, w[(size_t)q * ldw], acc[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-      if (q < jn) Cm[k + (size_t)(j0 + q) * ldc] = acc[q];
-  }
-  __syncthreads();
 }
 
 // W <- T^T W (trans) or T W in place, T an ib x ib upper triangle (leading
@@ -468,6 +516,58 @@ __device__ void trmm_tw(Real *W, int ldw, const Real *Tq, int ldq, int ib, int N
     if (on) {
       w[ra] = sa;
       w[rb] = sb;
+    }
+  }
+  __syncthreads();
+}
+
+// W2 <- T^T W (trans) or T W, out of place, and for TS / TT (ct: the identity top
+// block's rows of C) ct -= W2. T an ib x ib upper triangle, ib even. A thread
+// forms rows h and ib - 1 - h of a column, ib + 1 terms whatever h is, each in
+// ascending order.
+template <typename Real>
+__device__ void trmm_out(Real *W2, const Real *W, int ldw, const Real *Tq, int ldq, int ib, int Nj, int trans, Real *ct,
+                         int ldc) {
+  const int hb = ib / 2;
+  for (ColWalk w(hb); w.c < Nj; w.next()) {
+    const Real *x = W + (size_t)w.c * ldw;
+    const int ra = w.r, rb = ib - 1 - w.r;
+    // hb steps that every lane's long row has, and hb + 1 steps for the rest of both rows
+    Real sa = 0, sb = 0;
+    if (trans) {
+      const Real *ta = Tq + (size_t)ra * ldq, *tb = Tq + (size_t)rb * ldq;
+#pragma unroll 4
+      for (int l = 0; l < hb; ++l) sb = fma(tb[l], x[l], sb);
+      const int nb2 = hb - ra;  // row rb: l = hb .. rb; then row ra: l = 0 .. ra
+#pragma unroll 4
+      for (int m = 0; m <= hb; ++m) {
+        const bool second = m < nb2;
+        const int l = second ? hb + m : m - nb2;
+        const Real tv = second ? tb[l] : ta[l];
+        const Real acc = fma(tv, x[l], second ? sb : sa);
+        if (second) sb = acc; else sa = acc;
+      }
+    } else {
+      const Real *ta = Tq + ra, *tb = Tq + rb;
+      const int na = hb - ra;  // row ra: l = ra .. hb - 1; then row rb: l = rb .. ib - 1
+#pragma unroll 4
+      for (int m = 0; m <= hb; ++m) {
+        const bool first = m < na;
+        const int l = first ? ra + m : rb + m - na;
+        const Real tv = first ? ta[(size_t)l * ldq] : tb[(size_t)l * ldq];
+        const Real acc = fma(tv, x[l], first ? sa : sb);
+        if (first) sa = acc; else sb = acc;
+      }
+#pragma unroll 4
+      for (int l = hb; l < ib; ++l) sa = fma(ta[(size_t)l * ldq], x[l], sa);
+    }
+    Real *y = W2 + (size_t)w.c * ldw;
+    y[ra] = sa;
+    y[rb] = sb;
+    if (ct) {
+      Real *d = ct + (size_t)w.c * ldc;
+      d[ra] -= sa;
+      d[rb] -= sb;
     }
   }
   __syncthreads();
@@ -774,6 +874,246 @@ __device__ void shape_v(Real *V, int ld, int L, int ncols, int mode, int coff, i
 template <typename Real>
 __host__ __device__ inline size_t engine_smem_bytes(int nb, int ib, int w, int wt, int vc);
 
+// Updates keep the whole reflector tile and its T in shared memory where that
+// leaves room for two CTAs per SM: tiles of 64 and smaller, FP32 tiles of 128
+// with slabs of 16 columns.
+constexpr size_t kResidentMax = 112 << 10;
+template <typename Real>
+__host__ __device__ inline size_t resident_smem_bytes(int nb, int ib, int w) {
+  const int lds = nb + smem_pad<Real>(), ldq = sizeof(Real) == 8 ? ib + smem_pad<Real>() : ib;
+  const size_t scr = sizeof(Real) == 8 ? NT : 16 * NT;
+  return sizeof(Real) * ((size_t)lds * (2 * w + nb) + (size_t)nb * ldq + 2 * (size_t)ib * w + scr);
+}
+template <typename Real>
+__host__ __device__ inline bool update_resident(int nb, int ib, int w) {
+  return resident_smem_bytes<Real>(nb, ib, w) <= kResidentMax;
+}
+
+// The three products of one block of a resident update, W = V^T C (+ Ct),
+// W2 = T^T W or T W (Ct -= W2) and C -= V W2, with IB the block's columns at
+// compile time (0: ib at run time; an integer division costs a thread about
+// as much as its share of a 16-column product).
+//
+// W(i,j): every thread takes one unit, in FP32 a 4 x 4 block of W over one of
+// up to 16 parts of the K rows (G parts, in FP64 one element and up to 4 parts);
+// the parts are summed in order through scr. `un` holds the thread's unit.
+struct TnUnit {
+  int mt, g, G;  // output (block), part, parts
+  bool on;
+};
+template <typename Real>
+__device__ __forceinline__ TnUnit tn_unit(int ib, int cw) {
+  const int T = sizeof(Real) == 8 ? ib * cw : ((ib + 3) >> 2) * ((cw + 3) >> 2);
+  TnUnit u;
+  u.G = max(1, min(sizeof(Real) == 8 ? 4 : 16, NT / T));
+  u.g = (int)threadIdx.x / T;
+  u.mt = (int)threadIdx.x - u.g * T;
+  u.on = u.g < u.G;
+  return u;
+}
+
+template <int IB>
+__device__ __forceinline__ void resident_tn(const TnUnit &un, float *W, const float *V, int lds, const float *Cm, int K,
+                                            int ib_, int Nj, const float *Ct, float *scr) {
+  const int ib = IB ? IB : ib_, ti = (ib + 3) >> 2, T = ti * ((Nj + 3) >> 2), G = un.G;
+  const int Kc = (((K + G - 1) / G) + 3) & ~3;
+  if (T * G <= NT) {
+    if (un.on) {
+      const int i0 = (un.mt % ti) * 4, j0 = (un.mt / ti) * 4;
+      float acc[4][4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+      const int k1 = min(K, (un.g + 1) * Kc);
+      const float *vp[4], *cp[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) vp[a] = V + min(i0 + a, ib - 1) * lds;
+#pragma unroll
+      for (int b = 0; b < 4; ++b) cp[b] = Cm + min(j0 + b, Nj - 1) * lds;
+#pragma unroll 2
+      for (int k = un.g * Kc; k < k1; k += 4) {
+        float4 v4[4], c4[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) v4[a] = *reinterpret_cast<const float4 *>(vp[a] + k);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) c4[b] = *reinterpret_cast<const float4 *>(cp[b] + k);
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            acc[a][b] = fmaf(v4[a].x, c4[b].x, acc[a][b]);
+            acc[a][b] = fmaf(v4[a].y, c4[b].y, acc[a][b]);
+            acc[a][b] = fmaf(v4[a].z, c4[b].z, acc[a][b]);
+            acc[a][b] = fmaf(v4[a].w, c4[b].w, acc[a][b]);
+          }
+      }
+      // row a of the block at (a T G + unit) * 4: consecutive threads, consecutive 16 bytes
+      float4 *dst = reinterpret_cast<float4 *>(scr) + un.g * T + un.mt;
+#pragma unroll
+      for (int a = 0; a < 4; ++a) dst[a * T * G] = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+    }
+    __syncthreads();
+    for (int o = threadIdx.x; o < ib * Nj; o += NT) {
+      const int i = o % ib, j = o / ib;
+      const float *q = scr + ((i & 3) * T * G + (i >> 2) + (j >> 2) * ti) * 4 + (j & 3);
+      float s = Ct ? Ct[i + j * lds] : 0.f;
+      float r = 0.f;
+#pragma unroll 4
+      for (int g = 0; g < G; ++g) r += q[g * T * 4];
+      W[o] = s + r;
+    }
+    __syncthreads();
+  } else {
+    gemm_tn(W, ib, V, lds, Cm, lds, K, ib, Nj, Ct, lds, scr);
+  }
+}
+
+template <int IB>
+__device__ __forceinline__ void resident_tn(const TnUnit &un, double *W, const double *V, int lds, const double *Cm, int K,
+                                            int ib_, int Nj, const double *Ct, double *scr) {
+  const int ib = IB ? IB : ib_, T = ib * Nj, G = un.G;
+  const int Kc = (K + G - 1) / G;
+  for (int o = G > 1 ? un.mt : (int)threadIdx.x; o < T; o += NT) {
+    const int i = o % ib, j = o / ib;
+    const double *v = V + i * lds, *c = Cm + j * lds;
+    const int k1 = G > 1 ? min(K, (un.g + 1) * Kc) : K;
+    double s0 = 0, s1 = 0;
+    int k = G > 1 ? un.g * Kc : 0;
+    if (G > 1 && !un.on) k = k1;
+#pragma unroll 2
+    for (; k + 3 < k1; k += 4) {
+      const double v0 = v[k], v1 = v[k + 1], v2 = v[k + 2], v3 = v[k + 3];
+      const double c0 = c[k], c1 = c[k + 1], c2 = c[k + 2], c3 = c[k + 3];
+      s0 = fma(v0, c0, s0);
+      s1 = fma(v1, c1, s1);
+      s0 = fma(v2, c2, s0);
+      s1 = fma(v3, c3, s1);
+    }
+    for (; k < k1; ++k) s0 = fma(v[k], c[k], s0);
+    if (G > 1) {
+      if (un.on) scr[un.g * T + o] = s0 + s1;
+      break;
+    }
+    W[o] = (Ct ? Ct[i + j * lds] : 0.0) + (s0 + s1);
+  }
+  __syncthreads();
+  if (G > 1) {
+    if ((int)threadIdx.x < T) {
+      const int o = threadIdx.x, i = o % ib, j = o / ib;
+      double s = Ct ? Ct[i + j * lds] : 0.0;
+      for (int g = 0; g < G; ++g) s += scr[g * T + o];
+      W[o] = s;
+    }
+    __syncthreads();
+  }
+}
+
+// C -= V W2. FP32: lanes along k in fours, CH columns per thread; as many lanes
+// as the rows need (a power of two) share a column group.
+template <int IB, int CH>
+__device__ __forceinline__ void resident_nn(float *Cm, int lds, const float *V, const float *W, int K, int ib_, int Nj) {
+  const int ib = IB ? IB : ib_;
+  const int lg = K > 64 ? 5 : (K > 32 ? 4 : 3), kl = (int)threadIdx.x & ((1 << lg) - 1);
+  for (int j0 = ((int)threadIdx.x >> lg) * CH; j0 < Nj; j0 += (NT >> lg) * CH)
+    for (int k0 = kl * 4; k0 < K; k0 += 4 << lg) {
+      float4 acc[CH];
+#pragma unroll
+      for (int b = 0; b < CH; ++b) acc[b] = make_float4(0.f, 0.f, 0.f, 0.f);
+      const float *w = W + j0 * ib;
+#pragma unroll(CH == 2 ? 8 : 2)
+      for (int i = 0; i < ib; ++i) {
+        const float4 v = *reinterpret_cast<const float4 *>(V + i * lds + k0);
+#pragma unroll
+        for (int b = 0; b < CH; ++b) {
+          const float x = j0 + b < Nj ? w[b * ib + i] : 0.f;
+          acc[b].x = fmaf(v.x, x, acc[b].x);
+          acc[b].y = fmaf(v.y, x, acc[b].y);
+          acc[b].z = fmaf(v.z, x, acc[b].z);
+          acc[b].w = fmaf(v.w, x, acc[b].w);
+        }
+      }
+#pragma unroll
+      for (int b = 0; b < CH; ++b)
+        if (j0 + b < Nj) {
+          float4 *c = reinterpret_cast<float4 *>(Cm + (j0 + b) * lds + k0);
+          float4 x = *c;
+          x.x -= acc[b].x;
+          x.y -= acc[b].y;
+          x.z -= acc[b].z;
+          x.w -= acc[b].w;
+          *c = x;
+        }
+    }
+  __syncthreads();
+}
+template <int IB>
+__device__ __forceinline__ void resident_nn(float *Cm, int lds, const float *V, const float *W, int K, int ib, int Nj) {
+  if (Nj <= 16)
+    resident_nn<IB, 2>(Cm, lds, V, W, K, ib, Nj);
+  else
+    resident_nn<IB, 8>(Cm, lds, V, W, K, ib, Nj);
+}
+template <int IB>
+__device__ __forceinline__ void resident_nn(double *Cm, int lds, const double *V, const double *W, int K, int ib, int Nj) {
+  gemm_nn_sub(Cm, lds, V, lds, W, IB ? IB : ib, K, IB ? IB : ib, Nj);
+}
+
+// An update with everything it reads staged at once: C, the reflector tile and
+// all blocks of T. The blocks then follow each other without a copy to wait
+// for (the block-wise staging below costs a task about 2 us per block), with
+// the products of resident_tn / resident_nn. One TS task: 128 x 128 FP32 tiles,
+// 16 columns, blocks of 16: 45 -> 20 us; 64 x 64 FP64, 4 columns: 31 -> 19 us.
+template <typename Real, int IB>
+__device__ void task_update_resident(const EngineParams &p, const Geo<Real> &g, const Task &t, Shared<Real> &sh,
+                                     Real *dyn, uint32_t &phase) {
+  const int nb = g.nb, ib = IB ? IB : g.ib, lds = g.lds, cw = t.cw;
+  const int wmax = t.tgt == 0 ? g.w : g.wb;
+  const int ldq = sizeof(Real) == 8 ? g.ldt : ib;
+  Real *C1 = dyn;
+  Real *C2 = C1 + (size_t)lds * wmax;
+  Real *V = C2 + (size_t)lds * wmax;
+  Real *Tq = V + (size_t)lds * nb;
+  Real *W = Tq + (size_t)nb * ldq;
+  Real *W2 = W + (size_t)ib * wmax;
+  Real *scr = W2 + (size_t)ib * wmax;
+  const int op = t.op;
+  const bool pair = op != OP_UNMQR;
+  Real *g1 = g.target(t, pair ? t.r : t.i);
+  Real *g2 = pair ? g.target(t, t.i) : nullptr;
+  {
+    Copy<Real> cp[4] = {{C1, lds, g1, nb, nb, cw},
+                        {C2, lds, g2, nb, pair ? nb : 0, cw},
+                        {V, lds, g.tile(t.i, t.k), nb, nb, nb},
+                        {Tq, ldq, g.tfac(pair ? 1 : 0, t.i, t.k), ib, ib, nb}};
+    stage(p, sh, cp, 4, phase);
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (op != OP_TSMQR) {  // GE: unit lower triangle, TT: upper triangle
+    for (int c = warp; c < nb; c += NWARP) {
+      Real *v = V + (size_t)c * lds;
+      if (op == OP_UNMQR)
+        for (int k = lane; k <= c; k += 32) v[k] = k == c ? Real(1) : Real(0);
+      else
+        for (int k = c + 1 + lane; k < nb; k += 32) v[k] = 0;
+    }
+    __syncthreads();
+  }
+  const TnUnit un = tn_unit<Real>(ib, cw);
+  const int nq = nb / ib;
+  for (int qq = 0; qq < nq; ++qq) {
+    const int q = t.trans ? qq : nq - 1 - qq, q0 = q * ib;
+    const int r0 = op == OP_UNMQR ? q0 : 0, L = op == OP_UNMQR ? nb - q0 : (op == OP_TSMQR ? nb : q0 + ib);
+    Real *Cb = pair ? C2 : C1 + q0, *Ct = C1 + q0;
+    const Real *Vq = V + (size_t)q0 * lds + r0;
+    resident_tn<IB>(un, W, Vq, lds, Cb, L, ib, cw, pair ? Ct : (const Real *)nullptr, scr);
+    trmm_out(W2, W, ib, Tq + (size_t)q0 * ldq, ldq, ib, cw, t.trans, pair ? Ct : (Real *)nullptr, lds);
+    resident_nn<IB>(Cb, lds, Vq, W2, L, ib, cw);
+  }
+  store_cols(g1, nb, C1, lds, nb, cw, 0, 0);
+  if (pair) store_cols(g2, nb, C2, lds, nb, cw, 0, 0);
+}
+
 // Updates UNMQR / TSMQR / TTMQR of one column slab (also used for Q and Q^T
 // applied to right-hand-side blocks). V is staged in chunks of columns; the
 // chunk buffer comes last in shared memory and may use what the panel tasks
@@ -787,13 +1127,21 @@ __device__ void task_update(const EngineParams &p, const Geo<Real> &g, const Tas
                             Real *dyn, uint32_t &phase) {
   const int nb = g.nb, ib = g.ib, lds = g.lds, cw = t.cw;
   const int wmax = t.tgt == 0 ? g.w : g.wb;
+  if (t.blk == 0 && update_resident<Real>(nb, ib, wmax)) {
+    if (ib == 16)
+      task_update_resident<Real, 16>(p, g, t, sh, dyn, phase);
+    else
+      task_update_resident<Real, 0>(p, g, t, sh, dyn, phase);
+    return;
+  }
   const int VC = g.vc;
   Real *C1 = dyn;
   Real *C2 = C1 + (size_t)lds * wmax;
   const int ldq = sizeof(Real) == 8 ? g.ldt : ib;  // T of the block (FP64: padded for the paired trmm)
   Real *Tq = C2 + (size_t)lds * wmax;
   Real *W = Tq + (size_t)ib * ldq;
-  Real *scr = W + (size_t)ib * wmax;
+  Real *W2 = W + (size_t)ib * wmax;
+  Real *scr = W2 + (size_t)ib * wmax;
   const size_t su = (sizeof(Real) == 4 ? 4 : 1) * (size_t)(((VC + 3) / 4) * ((wmax + 3) / 4) * 16);
   Real *Vc = scr + (su > (size_t)NT ? su : (size_t)NT);
   const size_t vcap = engine_smem_bytes<Real>(nb, ib, g.w > g.wb ? g.w : g.wb, g.wt, VC) / sizeof(Real) -
@@ -832,8 +1180,7 @@ __device__ void task_update(const EngineParams &p, const Geo<Real> &g, const Tas
       shape_v(Vc, ldv, L, vq, mode, c * vq, q0);
       gemm_tn(W + c * vq, ib, Vc, ldv, Cb, lds, L, vq, cw, pair ? Ct + c * vq : nullptr, lds, scr);
     }
-    trmm_tw(W, ib, Tq, ldq, ib, cw, t.trans);
-    if (pair) sub_top(Ct, lds, W, ib, ib, cw);
+    trmm_out(W2, W, ib, Tq, ldq, ib, cw, t.trans, pair ? Ct : (Real *)nullptr, lds);
     for (int c = 0; c < nchunk; ++c) {
       if (nchunk > 1) {
         __syncthreads();
@@ -841,7 +1188,7 @@ __device__ void task_update(const EngineParams &p, const Geo<Real> &g, const Tas
         stage(p, sh, cp, 1, phase);
         shape_v(Vc, ldv, L, vq, mode, c * vq, q0);
       }
-      gemm_nn_sub(Cb, lds, Vc, ldv, W + c * vq, ib, L, vq, cw);
+      gemm_nn_sub(Cb, lds, Vc, ldv, W2 + c * vq, ib, L, vq, cw);
     }
   }
   store_cols(g1, nb, C1, lds, nb, cw, 0, 0);
@@ -2005,12 +2352,14 @@ __host__ __device__ inline size_t engine_smem_bytes(int nb, int ib, int w, int w
   const size_t sp = sp1 > sp2 ? sp1 : sp2;
   const size_t scr_p = sp > (size_t)NT ? sp : (size_t)NT;
   const int ldq = sizeof(Real) == 8 ? ldt : ib;  // T of a block
-  const size_t upd = (size_t)lds * (2 * w + vc) + (size_t)ib * ldq + (size_t)ib * w + scr_u;
+  const size_t upd = (size_t)lds * (2 * w + vc) + (size_t)ib * ldq + 2 * (size_t)ib * w + scr_u;
   const size_t cbg = (size_t)(lds * wt > ib * ib ? lds * wt : ib * ib);
   const size_t pan = (size_t)lds * ib + (size_t)ldt * (ib + wt) + (size_t)ib * ldq + cbg +
                      (size_t)ib * wt + scr_p;
   const size_t vec = (size_t)(2 * NT + 256) * sizeof(double);  // FP64 vector tasks
-  const size_t tiles = sizeof(Real) * (upd > pan ? upd : pan);
+  size_t tiles = sizeof(Real) * (upd > pan ? upd : pan);
+  if (update_resident<Real>(nb, ib, w) && resident_smem_bytes<Real>(nb, ib, w) > tiles)
+    tiles = resident_smem_bytes<Real>(nb, ib, w);
   return tiles > vec ? tiles : vec;
 }
 

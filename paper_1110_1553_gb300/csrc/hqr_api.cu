@@ -206,9 +206,13 @@ const void *sched_kernel(int prec, bool tc) {
 
 size_t smem_for(int prec, const Problem &P) {
   if (P.tc) return engine_smem_bytes_tc();
-  const int wmax = std::max(P.w, P.wb);
-  return prec == HQR_FP64 ? engine_smem_bytes<double>(P.nb, P.ib, wmax, P.wt, P.vc)
-                          : engine_smem_bytes<float>(P.nb, P.ib, wmax, P.wt, P.vc);
+  // tile slabs (w columns) and right-hand-side blocks (wb): one may keep the reflector tile resident
+  // where the other does not
+  auto bytes = [&](int w) {
+    return prec == HQR_FP64 ? engine_smem_bytes<double>(P.nb, P.ib, w, P.wt, P.vc)
+                            : engine_smem_bytes<float>(P.nb, P.ib, w, P.wt, P.vc);
+  };
+  return std::max(bytes(P.w), bytes(P.wb));
 }
 
 // CTAs for a launch: every SM filled to the occupancy the kernel allows.
@@ -2786,14 +2790,9 @@ extern "C" int hqr_geqrf_r_noalloc(const void *dA, int M, int N, int lda, int nb
   p.ctl = dctl;
   p.timeout_ns = g_timeout_ns;
   const size_t smem = engine_smem_bytes<double>(nb, ib, w, wt, vc);
-  int sms = 0, per_sm = 0;
-  if (cudaFuncSetAttribute(hqr_sched<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-          cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hqr_sched<double, false>, NT, smem) != cudaSuccess ||
-      per_sm < 1)
-    return HQR_ERR_CUDA;
-  hqr_sched<double, false><<<std::max(1, std::min(sms * per_sm, nt)), NT, smem, s>>>(p);
+  int grid = 0;
+  if (ctas_for(HQR_FP64, false, smem, nt, &grid)) return HQR_ERR_CUDA;
+  hqr_sched<double, false><<<grid, NT, smem, s>>>(p);
   unpack_tiles<double><<<grid_for((long long)N * N), 256, 0, s>>>((const double *)dws, m, nb, (double *)dR, ldr, N,
                                                                  N, 1);
   if (cudaGetLastError() != cudaSuccess) return HQR_ERR_CUDA;

@@ -73,6 +73,13 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
       : "memory");
 }
 
+// 16 bytes global -> shared, asynchronous, read around L1; complete for this
+// thread after cp_async_wait_all (for the CTA after a barrier on top).
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // Dynamic shared memory of the running launch, in bytes.
 __device__ __forceinline__ uint32_t dynamic_smem_bytes() {
   uint32_t v;

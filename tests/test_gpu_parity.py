@@ -326,3 +326,35 @@ def test_panel_scaled_columns(shape, a, nb, ib, dtype):
     keep = scale != 0
     err = np.abs(R[:, keep] / scale[keep] - base[:, keep]) / np.linalg.norm(A, axis=0)[keep]
     assert np.max(err) <= (R_TOL if dtype == "f64" else 5e-6)
+
+
+@pytest.mark.parametrize("dtype,nb,ib,w", [("f64", 64, 32, 16), ("f64", 88, 8, 16), ("f64", 96, 16, 8), ("f64", 96, 16, 16),
+                                           ("f64", 104, 8, 4), ("f64", 40, 4, 4), ("f32", 128, 16, 16), ("f32", 128, 16, 12),
+                                           ("f32", 128, 32, 16), ("f32", 64, 8, 64), ("f32", 136, 8, 8)])
+def test_updates_on_both_sides_of_the_resident_limit(dtype, nb, ib, w):
+    """Update tasks with the reflector tile staged whole (small tiles, narrow
+    slabs) and block by block (the others), and right-hand sides of 1 and 19
+    columns, which may take the other way than the tiles: R, Q^T B and Q B
+    against the oracle, with TS and TT kernels and a ragged last tile."""
+    m, n = 4, 2
+    A = inputs.gaussian(m * nb - 5, n * nb - 3, seed=180 + nb + w)
+    recs = hqr_elim_list(m, n, 2, 1, GREEDY, GREEDY)
+    rt, bt = (R_TOL, 1e-12) if dtype == "f64" else (5e-6, 5e-6)
+    if dtype == "f32":
+        A = A.astype(np.float32).astype(np.float64)
+    Fo = tile_qr(pad(A, nb), nb, ib, recs)
+    Ad = torch.from_numpy(A).cuda()
+    hqr.set_slab_widths(w, 0, 0)
+    try:
+        F = hqr.geqrf(Ad if dtype == "f64" else Ad.float(), nb, ib, recs)
+    finally:
+        hqr.set_slab_widths(0, 0, 0)
+    N = A.shape[1]
+    assert np.max(np.abs(F.R().double().cpu().numpy() - np.triu(Fo.A[:N, :N]))) <= rt * np.linalg.norm(A)
+    for k in (1, 19):
+        B = pad(inputs.gaussian(A.shape[0], k, seed=181 + k).astype(np.float32).astype(np.float64), 1)
+        for trans in (True, False):
+            Bd = torch.from_numpy(B.copy()).cuda()
+            out = F.apply_q(Bd if dtype == "f64" else Bd.float(), trans=trans).double().cpu().numpy()
+            ref = o_apply_q(Fo, np.vstack([B, np.zeros((m * nb - B.shape[0], k))]), trans=trans)[:B.shape[0]]
+            assert np.max(np.abs(out - ref)) <= bt * np.linalg.norm(B)
