@@ -1301,6 +1301,57 @@ __device__ __forceinline__ void dot2_merge(double &s1, double &c1, double s2, do
   c1 += c2 + e;
 }
 
+// A compensated sum of products in four FP64 operations per term (Dot2 takes
+// ten): s starts at sig = 1.5 2^E and stays within 2^(E-1) of it, so in one
+// binade, and z = fl(s + a x) - s is exact; e = fl(a x - z) then holds what the
+// sum did not take, to 2^(E-106), and goes to c. The sum is (s - sig) + c.
+// Before each group of eight terms, E is raised (s moves to a larger sig, exactly) if
+// a product may exceed 2^(E-5) or s is further than 2^(E-2) from sig: E settles
+// a few binades above the largest product, where Dot2's error follows the
+// running sum's magnitude. Groups whose exponents leave the range take Dot2.
+struct BiasedSum {
+  double s = 0.0, c = 0.0, sig = 0.0;
+  int eb = 0;  // biased exponent of sig (0: none yet)
+  double fs = 0.0, fc = 0.0;
+  bool far = false;
+  __device__ __forceinline__ void raise(int neb) {
+    const double ns = __hiloint2double((neb << 20) | 0x80000, 0), q = s - sig, b = q + ns;
+    c += q - (b - ns);
+    s = b;
+    sig = ns;
+    eb = neb;
+  }
+  // biased exponents of a and x added up: |a x| < 2^(this - 2044)
+  __device__ __forceinline__ static int exponents(double a, double x) {
+    return ((__double2hiint(a) >> 20) & 0x7ff) + ((__double2hiint(x) >> 20) & 0x7ff);
+  }
+  __device__ __forceinline__ bool centred() const {
+    const int d = __double2hiint(s) - __double2hiint(sig);
+    return d < (1 << 18) && d > -(1 << 18);
+  }
+  // N <= 8 terms; m: their largest exponents(), ok: centred() (both over the warp where its lanes are to
+  // share sig)
+  template <int N>
+  __device__ __forceinline__ void terms(const double (&a)[N], const double (&x)[N], int m, bool ok) {
+    if (m - 1016 > eb || !ok) {
+      const int neb = max(m - 1015, eb + 1);
+      if (neb < 200 || neb > 1980) {
+        far = true;
+#pragma unroll
+        for (int u = 0; u < N; ++u) dot2_step(a[u], x[u], fs, fc);
+        return;
+      }
+      raise(neb);
+    }
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+      const double n = fma(a[u], x[u], s), z = n - s;
+      c += fma(a[u], x[u], -z);
+      s = n;
+    }
+  }
+};
+
 // sum over q = q0, q0 + step, ... < q1 of M(q, o) g_q (transposed) or M(o, q) g_q, M column-major
 // with leading dimension ld (in shared memory when staged, else global: M is final for the whole
 // launch, R tiles after their factorization, the inverses after their TRINV task), in FP64 with
@@ -1430,40 +1481,48 @@ __device__ void task_vector(const EngineParams &p, const Problem &P, const Geo<R
         for (; j < chi; j += G) s = fma(ptx::to_f64(__ldcg(arow + (long long)j * P.lda0)), __ldcg(P.x + j), s);
         s = (s + s1) + (s2 + s3);
       } else if (rr < nr && gi < G) {
-        // four independent compensated sums (more FP64 work in flight), merged in a fixed order
+        // groups of eight columns (the same for every KU), KU in flight
         const Real *arow = A0 + r0 + rr;
-        double s1 = 0.0, c1 = 0.0, s2 = 0.0, c2 = 0.0, s3 = 0.0, c3 = 0.0;
+        BiasedSum d;
+        auto group = [&](const Real(&a)[8], const double(&xv)[8]) {
+          double av[8];
+          int m = 0;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            av[u] = ptx::to_f64(a[u]);
+            m = max(m, BiasedSum::exponents(av[u], xv[u]));
+          }
+          d.terms(av, xv, m, d.centred());
+        };
         int j = clo + gi;
-        for (; j + (KU - 1) * G < chi; j += KU * G) {  // KU columns in flight, the same order per sum
-          Real a[KU];
-          double xv[KU];
+        for (; j + (KU - 1) * G < chi; j += KU * G) {
+          Real a[KU / 8][8];
+          double xv[KU / 8][8];
 #pragma unroll
           for (int u = 0; u < KU; ++u) {
+            a[u / 8][u % 8] = __ldcg(arow + (long long)(j + u * G) * P.lda0);
+            xv[u / 8][u % 8] = __ldcg(P.x + j + u * G);
+          }
+#pragma unroll
+          for (int h = 0; h < KU / 8; ++h) group(a[h], xv[h]);
+        }
+        for (; KU > 8 && j + 7 * G < chi; j += 8 * G) {
+          Real a[8];
+          double xv[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
             a[u] = __ldcg(arow + (long long)(j + u * G) * P.lda0);
             xv[u] = __ldcg(P.x + j + u * G);
           }
-#pragma unroll
-          for (int u = 0; u < KU; u += 4) {
-            dot2_step(ptx::to_f64(a[u]), xv[u], s, c);
-            dot2_step(ptx::to_f64(a[u + 1]), xv[u + 1], s1, c1);
-            dot2_step(ptx::to_f64(a[u + 2]), xv[u + 2], s2, c2);
-            dot2_step(ptx::to_f64(a[u + 3]), xv[u + 3], s3, c3);
-          }
+          group(a, xv);
         }
-        for (; j + 3 * G < chi; j += 4 * G) {
-          const double a0 = ptx::to_f64(__ldcg(arow + (long long)j * P.lda0));
-          const double a1 = ptx::to_f64(__ldcg(arow + (long long)(j + G) * P.lda0));
-          const double a2 = ptx::to_f64(__ldcg(arow + (long long)(j + 2 * G) * P.lda0));
-          const double a3 = ptx::to_f64(__ldcg(arow + (long long)(j + 3 * G) * P.lda0));
-          dot2_step(a0, __ldcg(P.x + j), s, c);
-          dot2_step(a1, __ldcg(P.x + j + G), s1, c1);
-          dot2_step(a2, __ldcg(P.x + j + 2 * G), s2, c2);
-          dot2_step(a3, __ldcg(P.x + j + 3 * G), s3, c3);
+        for (; j < chi; j += G) {
+          const double a[1] = {ptx::to_f64(__ldcg(arow + (long long)j * P.lda0))}, xv[1] = {__ldcg(P.x + j)};
+          d.terms(a, xv, BiasedSum::exponents(a[0], xv[0]), d.centred());
         }
-        for (; j < chi; j += G) dot2_step(ptx::to_f64(__ldcg(arow + (long long)j * P.lda0)), __ldcg(P.x + j), s, c);
-        dot2_merge(s, c, s1, c1);
-        dot2_merge(s2, c2, s3, c3);
-        dot2_merge(s, c, s2, c2);
+        s = d.s - d.sig;
+        c = d.c;
+        if (d.far) dot2_merge(s, c, d.fs, d.fc);
       }
       sm[tid] = s;
       sm[NT + tid] = c;
@@ -1527,7 +1586,7 @@ __device__ void task_vector(const EngineParams &p, const Problem &P, const Geo<R
       const size_t np = (size_t)g.n * nb;
       for (int cc = warp; cc < nc; cc += NWARP) {
         const Real *acol = A0 + (long long)(c0 + cc) * P.lda0;
-        double s = 0.0, c = 0.0, s1 = 0.0, c1 = 0.0, s2 = 0.0, c2 = 0.0, s3 = 0.0, c3 = 0.0;
+        double s = 0.0, c = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
         int i = rlo + lane;
         if (!comp) {  // plain FP64 round: FMA chains, then a plain warp sum
           for (; i + 32 * (KU - 1) < rhi; i += 32 * KU) {  // KU rows in flight, the same order per chain
@@ -1560,38 +1619,48 @@ __device__ void task_vector(const EngineParams &p, const Problem &P, const Geo<R
           }
           continue;
         }
-        for (; i + 32 * (KU - 1) < rhi; i += 32 * KU) {  // KU rows in flight, the same order per sum
-          Real a[KU];
-          double rv[KU];
+        // the lanes share sig, so that their high parts, multiples of one unit, add up exactly once sig has
+        // five more binades of room
+        BiasedSum d;
+        auto group = [&](const Real(&a)[8], const double(&rv)[8]) {
+          double av[8];
+          int m = 0;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            av[u] = ptx::to_f64(a[u]);
+            m = max(m, BiasedSum::exponents(av[u], rv[u]));
+          }
+          d.terms(av, rv, (int)__reduce_max_sync(0xffffffffu, (unsigned)m), __all_sync(0xffffffffu, d.centred()));
+        };
+        for (int k = rlo; k < rhi; k += 32 * KU) {
+          Real a[KU / 8][8];
+          double rv[KU / 8][8];
 #pragma unroll
           for (int u = 0; u < KU; ++u) {
-            a[u] = __ldcg(acol + i + 32 * u);
-            rv[u] = __ldcg(P.r + i + 32 * u);
+            const int row = k + lane + 32 * u;
+            a[u / 8][u % 8] = row < rhi ? __ldcg(acol + row) : Real(0);
+            rv[u / 8][u % 8] = row < rhi ? __ldcg(P.r + row) : 0.0;
           }
 #pragma unroll
-          for (int u = 0; u < KU; u += 4) {
-            dot2_step(ptx::to_f64(a[u]), rv[u], s, c);
-            dot2_step(ptx::to_f64(a[u + 1]), rv[u + 1], s1, c1);
-            dot2_step(ptx::to_f64(a[u + 2]), rv[u + 2], s2, c2);
-            dot2_step(ptx::to_f64(a[u + 3]), rv[u + 3], s3, c3);
-          }
+          for (int h = 0; h < KU / 8; ++h)
+            if (k + 32 * 8 * h < rhi) group(a[h], rv[h]);
         }
-        for (; i + 96 < rhi; i += 128) {  // four independent compensated sums, merged in a fixed order
-          const double a0 = ptx::to_f64(__ldcg(acol + i)), a1 = ptx::to_f64(__ldcg(acol + i + 32));
-          const double a2 = ptx::to_f64(__ldcg(acol + i + 64)), a3 = ptx::to_f64(__ldcg(acol + i + 96));
-          dot2_step(a0, __ldcg(P.r + i), s, c);
-          dot2_step(a1, __ldcg(P.r + i + 32), s1, c1);
-          dot2_step(a2, __ldcg(P.r + i + 64), s2, c2);
-          dot2_step(a3, __ldcg(P.r + i + 96), s3, c3);
-        }
-        for (; i < rhi; i += 32) dot2_step(ptx::to_f64(__ldcg(acol + i)), __ldcg(P.r + i), s, c);
-        dot2_merge(s, c, s1, c1);
-        dot2_merge(s2, c2, s3, c3);
-        dot2_merge(s, c, s2, c2);
+        d.raise(d.eb + 5);
+        s = d.s - d.sig;
+        c = d.c;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-          const double s2 = __shfl_xor_sync(0xffffffffu, s, o), c2 = __shfl_xor_sync(0xffffffffu, c, o);
-          dot2_merge(s, c, s2, c2);
+          s += __shfl_xor_sync(0xffffffffu, s, o);
+          c += __shfl_xor_sync(0xffffffffu, c, o);
+        }
+        if (d.far) {  // the same in every lane
+          double fs = d.fs, fc = d.fc;
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            const double s2 = __shfl_xor_sync(0xffffffffu, fs, o), c2 = __shfl_xor_sync(0xffffffffu, fc, o);
+            dot2_merge(fs, fc, s2, c2);
+          }
+          dot2_merge(s, c, fs, fc);
         }
         if (lane == 0) {
           P.gp[2 * ((size_t)t.i * np + c0 + cc)] = s;

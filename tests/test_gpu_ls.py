@@ -135,3 +135,21 @@ def test_mixed_square_conditioned_matches_oracle(kappa, iters):
     plan2 = hqr.LSPlan([(A, b, x2)], refine_iters=2, configs=[hqr.tile_config(128, 16, 4, 1)])
     plan2.run()
     assert plan2.status() == 0 and plan2.correction(0) > 1e-9
+
+
+@pytest.mark.parametrize("M,N,nb", [(300, 40, 32), (1100, 129, 64), (700, 260, 128), (65, 65, 64)])
+@pytest.mark.parametrize("tensor", [False, True])
+def test_refinement_with_graded_columns(M, N, nb, tensor):
+    """Compensated residuals and A^T r over products of very different sizes:
+    columns of an FP32 matrix scaled by powers of two from 2^-40 to 2^40 (exact)
+    scale x by the inverse, so x times the scale must meet the oracle's
+    solution of the unscaled problem within the refinement's 1e-12."""
+    A, b = make(M, N, 90 + N, np.float32)
+    scale = np.ldexp(1.0, np.random.default_rng(N).integers(-40, 41, N))
+    xo = lstsq_unblocked(A.astype(np.float64), b)
+    pr = to_dev((A * scale).astype(np.float32), b, N)
+    plan = hqr.LSPlan([pr], refine_iters=12, configs=[hqr.tile_config(nb, min(16, nb), 2, 1)], tensor=tensor)
+    plan.run()
+    assert plan.status() == 0
+    err = np.linalg.norm(pr[2].cpu().numpy() * scale - xo) / np.linalg.norm(xo)
+    assert err <= 1e-12, err
