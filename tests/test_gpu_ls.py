@@ -153,3 +153,18 @@ def test_refinement_with_graded_columns(M, N, nb, tensor):
     assert plan.status() == 0
     err = np.linalg.norm(pr[2].cpu().numpy() * scale - xo) / np.linalg.norm(xo)
     assert err <= 1e-12, err
+
+
+@pytest.mark.parametrize("N,nb,ib", [(1, 32, 16), (31, 32, 16), (33, 40, 8), (72, 72, 8), (100, 256, 32), (257, 256, 32), (200, 136, 8)])
+@pytest.mark.parametrize("mixed", [False, True])
+def test_diagonal_tile_inverses(N, nb, ib, mixed):
+    """Inverses of diagonal R tiles by blocks of 32: tiles of one partial block
+    up to eight blocks, and a last tile whose leading part ends in any block."""
+    A, b = make(2 * N + 40, N, 300 + N, np.float32 if mixed else np.float64)
+    pr = to_dev(A, b, N)
+    plan = hqr.LSPlan([pr], refine_iters=8 if mixed else 0, configs=[hqr.tile_config(nb, ib, 2, 1)])
+    plan.run()
+    assert plan.status() == 0
+    xo = lstsq_unblocked(A.astype(np.float64), b)
+    err = np.linalg.norm(pr[2].cpu().numpy() - xo) / np.linalg.norm(xo)
+    assert err <= (1e-12 if mixed else 1e-13 * np.linalg.cond(A)), err
