@@ -33,25 +33,35 @@ bool cuda_ok(cudaError_t e, const char *what) {
     if (!cuda_ok((call), #call)) return HQR_ERR_CUDA; \
   } while (0)
 
-// A task graph resident on the device, with pristine copies of the
-// in-degrees, the ready slots and the control words for every new run.
+// Offsets of the parts of one device allocation (256-byte aligned).
+struct Layout {
+  size_t total = 0;
+  size_t add(size_t bytes) {
+    const size_t at = total;
+    total += (bytes + 255) & ~(size_t)255;
+    return at;
+  }
+};
+
+// A task graph resident on the device, in one allocation: tasks, successors,
+// and the in-degrees, ready slots and control words twice, as every run starts
+// with them and as the run changes them (each three in one piece, so that a
+// run resets them with one copy).
 struct DevGraph {
+  unsigned char *base = nullptr;
   Task *tasks = nullptr;
   int *succ = nullptr;
   int *indeg0 = nullptr, *indeg = nullptr;
-  int *slots0 = nullptr, *slots = nullptr;
-  Ctl *ctl0 = nullptr, *ctl = nullptr;
+  int *slots = nullptr;
+  Ctl *ctl = nullptr;
+  size_t run_bytes = 0;
   int ntasks = 0;
   int64_t nedges = 0;
+  cudaError_t reset(cudaStream_t s) const {
+    return cudaMemcpyAsync(indeg, indeg0, run_bytes, cudaMemcpyDeviceToDevice, s);
+  }
   void release() {
-    cudaFree(tasks);
-    cudaFree(succ);
-    cudaFree(indeg0);
-    cudaFree(indeg);
-    cudaFree(slots0);
-    cudaFree(slots);
-    cudaFree(ctl0);
-    cudaFree(ctl);
+    cudaFree(base);
     *this = DevGraph();
   }
 };
@@ -73,21 +83,39 @@ int upload_graph(const Graph &g, DevGraph &d) {
   std::vector<Ctl> ctlv(1);
   Ctl &ctl = ctlv[0];
   init_ready(g.tasks.data(), g.indeg.data(), nt, slots.data(), ctl);
-  const size_t ns = std::max<size_t>(g.succ.size(), 1);
-  CK(cudaMalloc(&d.tasks, sizeof(Task) * nt));
-  CK(cudaMalloc(&d.succ, sizeof(int) * ns));
-  CK(cudaMalloc(&d.indeg0, sizeof(int) * nt));
-  CK(cudaMalloc(&d.indeg, sizeof(int) * nt));
-  CK(cudaMalloc(&d.slots0, sizeof(int) * slots.size()));
-  CK(cudaMalloc(&d.slots, sizeof(int) * slots.size()));
-  CK(cudaMalloc(&d.ctl0, sizeof(Ctl)));
-  CK(cudaMalloc(&d.ctl, sizeof(Ctl)));
-  CK(cudaMemcpy(d.tasks, g.tasks.data(), sizeof(Task) * nt, cudaMemcpyHostToDevice));
-  if (!g.succ.empty())
-    CK(cudaMemcpy(d.succ, g.succ.data(), sizeof(int) * g.succ.size(), cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(d.indeg0, g.indeg.data(), sizeof(int) * nt, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(d.slots0, slots.data(), sizeof(int) * slots.size(), cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(d.ctl0, &ctl, sizeof(Ctl), cudaMemcpyHostToDevice));
+  Layout run;
+  const size_t r_indeg = run.add(sizeof(int) * nt), r_slots = run.add(sizeof(int) * slots.size()),
+               r_ctl = run.add(sizeof(Ctl));
+  Layout all;
+  const size_t o_tasks = all.add(sizeof(Task) * nt), o_succ = all.add(sizeof(int) * std::max<size_t>(g.succ.size(), 1)),
+               o_run0 = all.add(run.total), upload = all.total, o_run = all.add(run.total);
+  CK(cudaMalloc(&d.base, all.total));
+  d.tasks = (Task *)(d.base + o_tasks);
+  d.succ = (int *)(d.base + o_succ);
+  d.indeg0 = (int *)(d.base + o_run0 + r_indeg);
+  d.indeg = (int *)(d.base + o_run + r_indeg);
+  d.slots = (int *)(d.base + o_run + r_slots);
+  d.ctl = (Ctl *)(d.base + o_run + r_ctl);
+  d.run_bytes = run.total;
+  struct Part {
+    size_t at;
+    const void *src;
+    size_t bytes;
+  };
+  const Part parts[] = {{o_tasks, g.tasks.data(), sizeof(Task) * nt},
+                        {o_succ, g.succ.data(), sizeof(int) * g.succ.size()},
+                        {o_run0 + r_indeg, g.indeg.data(), sizeof(int) * nt},
+                        {o_run0 + r_slots, slots.data(), sizeof(int) * slots.size()},
+                        {o_run0 + r_ctl, &ctl, sizeof(Ctl)}};
+  if (upload <= ((size_t)4 << 20)) {  // a small graph goes up in one copy
+    std::vector<unsigned char> host(upload, 0);
+    for (const Part &q : parts)
+      if (q.bytes) std::memcpy(host.data() + q.at, q.src, q.bytes);
+    CK(cudaMemcpy(d.base, host.data(), upload, cudaMemcpyHostToDevice));
+  } else {
+    for (const Part &q : parts)
+      if (q.bytes) CK(cudaMemcpy(d.base + q.at, q.src, q.bytes, cudaMemcpyHostToDevice));
+  }
   return setup_done();
 }
 
@@ -391,9 +419,7 @@ int run_graph(hqr_factors *F, DevGraph &g, cudaStream_t s) {
   p.timeout_ns = g_timeout_ns;
   p.trace = (F->dtrace && F->trace_cap >= (size_t)g.ntasks) ? F->dtrace : nullptr;
   const size_t smem = smem_for(F->prec, F->prob);
-  CK(cudaMemcpyAsync(g.indeg, g.indeg0, sizeof(int) * g.ntasks, cudaMemcpyDeviceToDevice, s));
-  CK(cudaMemcpyAsync(g.slots, g.slots0, sizeof(int) * slot_count(g.ntasks), cudaMemcpyDeviceToDevice, s));
-  CK(cudaMemcpyAsync(g.ctl, g.ctl0, sizeof(Ctl), cudaMemcpyDeviceToDevice, s));
+  CK(g.reset(s));
   if (!F->ev0) {
     CK(cudaEventCreate(&F->ev0));
     CK(cudaEventCreate(&F->ev1));
@@ -1048,9 +1074,11 @@ struct hqr_ls_plan {
   std::vector<PrepDesc> prep;
   Problem *dprobs = nullptr;
   PrepDesc *dprep = nullptr;
+  unsigned char *mem = nullptr;  // the plan's one device allocation (but for graphs and traces): all of the below
   void *arena = nullptr;   // tiles, T, rhs blocks (storage precision)
   double *vec = nullptr;   // x, r, g of every problem
-  int *dstatus = nullptr;  // per-problem status words
+  int *dstatus = nullptr;  // per-problem status words, then drs
+  size_t state_bytes = 0;  // of both
   long long prep_total = 0;
   size_t smem = 0;
   double flops = 0.0;
@@ -1095,13 +1123,10 @@ int plan_enqueue(hqr_ls_plan *P, cudaStream_t s, bool timed) {
   else
     ls_prepare<float><<<grid_for(P->prep_total), 256, 0, s>>>(P->dprep, P->count, P->prep_total);
   CK(cudaGetLastError());
-  CK(cudaMemsetAsync(P->dstatus, 0, sizeof(int) * P->count, s));
-  if (P->drs) CK(cudaMemsetAsync(P->drs, 0, sizeof(RefineState) * P->count, s));
+  CK(cudaMemsetAsync(P->dstatus, 0, P->state_bytes, s));
   for (DevGraph *g : {&P->graph, &P->graph2}) {
     if (!g->ntasks) continue;
-    CK(cudaMemcpyAsync(g->indeg, g->indeg0, sizeof(int) * g->ntasks, cudaMemcpyDeviceToDevice, s));
-    CK(cudaMemcpyAsync(g->slots, g->slots0, sizeof(int) * slot_count(g->ntasks), cudaMemcpyDeviceToDevice, s));
-    CK(cudaMemcpyAsync(g->ctl, g->ctl0, sizeof(Ctl), cudaMemcpyDeviceToDevice, s));
+    CK(g->reset(s));
   }
   auto params = [&](const DevGraph &g, int tc, unsigned long long *trace) {
     EngineParams p{};
@@ -1246,12 +1271,23 @@ int plan_create(int count, const hqr_ls_problem_t *probs, const hqr_tile_config_
     P->flops += 2.0 * pr.M * (double)pr.N * pr.N - 2.0 / 3.0 * (double)pr.N * pr.N * pr.N;
   }
   int st = HQR_SUCCESS;
-  if (!cuda_ok(cudaMalloc(&P->arena, es * std::max<size_t>(arena_elems, 1)), "cudaMalloc(arena)") ||
-      !cuda_ok(cudaMalloc(&P->vec, sizeof(double) * std::max<size_t>(vec_elems, 1)), "cudaMalloc(vec)") ||
-      !cuda_ok(cudaMalloc(&P->dstatus, sizeof(int) * count), "cudaMalloc(status)") ||
-      (tol_mode && !cuda_ok(cudaMalloc(&P->drs, sizeof(RefineState) * count), "cudaMalloc(refine state)")) ||
-      !cuda_ok(cudaMemset(P->arena, 0, es * std::max<size_t>(arena_elems, 1)), "memset(arena)"))
+  Layout lay;
+  const size_t arena_bytes = es * std::max<size_t>(arena_elems, 1), o_arena = lay.add(arena_bytes),
+               o_vec = lay.add(sizeof(double) * std::max<size_t>(vec_elems, 1)),
+               o_probs = lay.add(sizeof(Problem) * count), o_prep = lay.add(sizeof(PrepDesc) * count),
+               o_status = lay.add(sizeof(int) * count), o_rs = lay.add(tol_mode ? sizeof(RefineState) * count : 0);
+  if (!cuda_ok(cudaMalloc(&P->mem, lay.total), "cudaMalloc(plan)") ||
+      !cuda_ok(cudaMemset(P->mem + o_arena, 0, arena_bytes), "memset(arena)")) {
     st = HQR_ERR_NOMEM;
+  } else {
+    P->arena = P->mem + o_arena;
+    P->vec = (double *)(P->mem + o_vec);
+    P->dprobs = (Problem *)(P->mem + o_probs);
+    P->dprep = (PrepDesc *)(P->mem + o_prep);
+    P->dstatus = (int *)(P->mem + o_status);
+    if (tol_mode) P->drs = (RefineState *)(P->mem + o_rs);
+    P->state_bytes = lay.total - o_status;
+  }
   if (!st) {
     long long off = 0;
     for (int q = 0; q < count; ++q) {
@@ -1287,9 +1323,6 @@ int plan_create(int count, const hqr_ls_problem_t *probs, const hqr_tile_config_
       P->prep.push_back(d);
     }
     P->prep_total = off;
-    if (!cuda_ok(cudaMalloc(&P->dprobs, sizeof(Problem) * count), "cudaMalloc(probs)") ||
-        !cuda_ok(cudaMalloc(&P->dprep, sizeof(PrepDesc) * count), "cudaMalloc(prep)"))
-      st = HQR_ERR_NOMEM;
   }
   if (!st && (!cuda_ok(cudaMemcpy(P->dprobs, P->probs.data(), sizeof(Problem) * count, cudaMemcpyHostToDevice),
                        "copy probs") ||
@@ -1572,12 +1605,7 @@ void hqr_ls_plan_free(hqr_ls_plan *P) {
     if (e) cudaEventDestroy(e);
   if (P->cge) cudaGraphExecDestroy(P->cge);
   if (P->cg) cudaGraphDestroy(P->cg);
-  cudaFree(P->arena);
-  cudaFree(P->vec);
-  cudaFree(P->dstatus);
-  cudaFree(P->drs);
-  cudaFree(P->dprobs);
-  cudaFree(P->dprep);
+  cudaFree(P->mem);
   cudaFree(P->dtrace);
   if (P->ev0) cudaEventDestroy(P->ev0);
   if (P->ev1) cudaEventDestroy(P->ev1);
