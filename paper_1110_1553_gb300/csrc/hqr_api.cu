@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -371,6 +372,19 @@ void choose_widths(int prec, int nb, int ib, Problem &P, long long tiles = 0) {
   if (g_vc_override > 0 && ib % g_vc_override == 0) P.vc = std::min(g_vc_override, ib);
 }
 
+// Columns of a right-hand-side block (one task of Q or Q^T on CUDA cores): the
+// replay is a chain of updates, so few row tiles and columns take narrow, short
+// tasks, many of them the cheaper wide ones. Times of Q in ms at 4 / 8 / 16
+// columns: FP64 8 tiles of 64, 512 columns 0.51 / 0.61 / 1.01, 2000 columns 1.71
+// / 1.31 / 1.31; 32 tiles of 128, 40 columns 2.5 / 2.9 / 4.8, 512 columns 12.2 /
+// 8.0 / 8.1; FP32 20 tiles of 128, 150 columns 0.72 / 0.74 / 0.97, 512 columns
+// 1.85 / 1.11 / 1.03.
+int rhs_width(int prec, bool tc, int nb, int m, int nrhs) {
+  const long long work = (long long)m * nrhs;
+  const int w = tc ? 16 : (work <= 4096 ? 4 : (work <= (prec == HQR_FP64 ? 16000 : 8192) ? 8 : 16));
+  return std::min(w, nb);
+}
+
 bool valid_tile_sizes(int prec, int nb, int ib) {
   if (use_tc(prec, nb)) return ib == nb;
   if (nb < 8 || nb > 256 || nb % 8) return false;
@@ -390,7 +404,7 @@ struct hqr_factors {
   void *dA = nullptr, *dT = nullptr, *dBw = nullptr;
   size_t bw_cap = 0;
   DevGraph fg;
-  std::map<std::pair<int, int>, DevGraph> ag;  // (trans, nslab) -> apply graph
+  std::map<std::array<int, 3>, DevGraph> ag;  // (trans, slabs, slab width) -> apply graph
   Ctl *last_ctl = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   bool timed = false;
@@ -801,21 +815,24 @@ int hqr_apply_q(hqr_factors *F, int trans, void *dB, int ldb, int nrhs, void *st
   if (nrhs == 0) return HQR_SUCCESS;
   g_launches = 0;
   cudaStream_t s = (cudaStream_t)stream;
-  const int wa = F->prob.wb;
+  const int wa = rhs_width(F->prec, F->prob.tc != 0, F->nb, F->m, nrhs);
   const int nslab = (nrhs + wa - 1) / wa;
   const size_t need = (size_t)F->Mp * nslab * wa;
   const size_t es = elem_size(F->prec);
-  if (need > F->bw_cap) {
+  if (need > F->bw_cap || wa != F->prob.wb) {
     CK(cudaStreamSynchronize(s));
-    cudaFree(F->dBw);
-    F->dBw = nullptr;
-    F->bw_cap = 0;
-    if (!cuda_ok(cudaMalloc(&F->dBw, es * need), "cudaMalloc(B)")) return HQR_ERR_NOMEM;
-    F->bw_cap = need;
+    if (need > F->bw_cap) {
+      cudaFree(F->dBw);
+      F->dBw = nullptr;
+      F->bw_cap = 0;
+      if (!cuda_ok(cudaMalloc(&F->dBw, es * need), "cudaMalloc(B)")) return HQR_ERR_NOMEM;
+      F->bw_cap = need;
+    }
+    F->prob.wb = wa;
     int st = push_problem(F);
     if (st) return st;
   }
-  auto key = std::make_pair(trans, nslab);
+  const std::array<int, 3> key = {trans, nslab, wa};
   auto it = F->ag.find(key);
   if (it == F->ag.end()) {
     Graph g = build_apply_graph(F->ops, F->m, nslab, wa, trans);

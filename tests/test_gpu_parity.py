@@ -358,3 +358,22 @@ def test_updates_on_both_sides_of_the_resident_limit(dtype, nb, ib, w):
             out = F.apply_q(Bd if dtype == "f64" else Bd.float(), trans=trans).double().cpu().numpy()
             ref = o_apply_q(Fo, np.vstack([B, np.zeros((m * nb - B.shape[0], k))]), trans=trans)[:B.shape[0]]
             assert np.max(np.abs(out - ref)) <= bt * np.linalg.norm(B)
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_apply_q_block_widths(dtype):
+    """Right-hand sides of sizes that take blocks of 4, 8 and 16 columns, in turn
+    on one factorization (the block layout changes between calls)."""
+    nb, ib, m, n = 16, 8, 40, 2
+    A = inputs.gaussian(m * nb, n * nb, seed=190).astype(np.float32).astype(np.float64)
+    recs = hqr_elim_list(m, n, 4, 2, GREEDY, BINARY)
+    Fo = tile_qr(A, nb, ib, recs)
+    Ad = torch.from_numpy(A).cuda()
+    F = hqr.geqrf(Ad if dtype == "f64" else Ad.float(), nb, ib, recs)
+    for k in (3, 110, 450, 102, 103, 5, 401):
+        B = inputs.gaussian(m * nb, k, seed=191 + k).astype(np.float32).astype(np.float64)
+        for trans in (True, False):
+            Bd = torch.from_numpy(B.copy()).cuda()
+            out = F.apply_q(Bd if dtype == "f64" else Bd.float(), trans=trans).double().cpu().numpy()
+            err = np.max(np.abs(out - o_apply_q(Fo, B, trans=trans)))
+            assert err <= (1e-12 if dtype == "f64" else 5e-6) * np.linalg.norm(B), (k, trans)
