@@ -335,15 +335,16 @@ void drop_t32(int prec, Problem &P) {
 // `tiles`: tiles of the factorization; 0 for plans and server requests, whose
 // launches hold other problems too and whose results must not depend on them
 // (the order of sums follows the width).
-// FP64 (ms, slabs of 16 / 8 / 4): 8 x 8 tiles of 64 2.66 / 2.52 / 2.40, 8 x 2
-// of 128 2.35 / 2.06 / 1.95, 16 x 16 of 64 6.1 / 5.7 / 6.0, 63 x 8 of 64 4.7 /
-// 5.3 / 8.0; inner blocks of 32 (more arithmetic per staged block): 16 x 16 of
-// 128 28.5 / 25.1 / 26.8, 32 x 16 of 128 47.8 / 42.7 / 57, 128 x 8 of 256
-// 259.5 / 255.5 (and 66 ms more on the host, so it stays at 16). FP32 on CUDA cores (slabs of 64 / 32 / 16): 20 x 14 of 128
-// 22.5 / 21.7 / 12.3 and 64 x 4 of 128 4.8 / 4.7 / 2.9 (slabs no wider than a
-// block also let the panels split, see split_ib_for), 10 x 5 of 64 1.29 / 1.25
-// / 1.10, 32 x 32 of 64 15.7 / 15.3 / 12.5 and of 128 47 / 46 / 29.5, 128 x 16 of
-// 128 29.8 / 29.2 / 35.7, 160 uneven problems 19.6 / 21.1 / 27.7.
+// FP64 (ms, slabs of 16 / 8 / 4): 8 x 8 tiles of 64 2.49 / 2.15 / 1.98, 8 x 2
+// of 128 2.40 / 1.94 / 1.83, 16 x 16 of 64 5.7 / 4.9 / 4.6 (4 doubles the tasks
+// the host builds), 63 x 8 of 64 4.3 / 4.0 / 4.9; inner blocks of 32 (more
+// arithmetic per staged block): 16 x 16 of 128 27.8 / 23.9 / 24.7, 32 x 16 of 128
+// 47 / 40 / 50, 128 x 8 of 256 259.5 / 255.5 (and 66 ms more on the host, so it
+// stays at 16). FP32 on CUDA cores (slabs of 64 / 32 / 16): 20 x 14 of 128 22.5 /
+// 17.7 / 10.1 and 64 x 4 of 128 4.8 / 3.8 / 2.4 (slabs no wider than a block also
+// let the panels split, see split_ib_for), 10 x 5 of 64 1.29 / 1.04 / 0.93, 128 x
+// 8 of 64 3.10 / 2.48 / 2.54, 32 x 32 of 128 47 / 46 / 29, 128 x 16 of 128 29.8 /
+// 29.2 / 35.7, 160 uneven problems 19.6 / 21.1 / 27.7.
 void choose_widths(int prec, int nb, int ib, Problem &P, long long tiles = 0) {
   P.wb = std::min(16, nb);
   P.tc = use_tc(prec, nb) ? 1 : 0;
