@@ -2396,8 +2396,12 @@ __device__ int serve_pop(const ServeParams &sp, unsigned &pending) {
   }
 }
 
+// The FP64 variant is held to 112 registers a thread, as it stays resident: with two CTAs of 256 on an
+// SM 8192 registers are left for the caller's kernels on other streams (fills, conversions). At 127
+// these, and a host thread behind them, waited for it to leave (2000 requests/s offered, with a fill per
+// submission: 80 to 113 solves/s, 134 now).
 template <typename Real, bool TC>
-__global__ void __launch_bounds__(NT, TC ? 1 : 2) hqr_serve(ServeParams sp) {
+__global__ void __maxnreg__(TC ? 255 : sizeof(Real) == 8 ? 112 : 128) hqr_serve(ServeParams sp) {
   extern __shared__ __align__(16) unsigned char dyn_raw[];
   Real *dyn = reinterpret_cast<Real *>(dyn_raw);
   __shared__ Shared<Real> sh;
