@@ -401,6 +401,8 @@ struct hqr_factors {
   std::vector<hqr_elim_t> list;
   std::vector<PanelOp> ops;
   Problem prob{};        // host copy of the device descriptor
+  // device descriptors: the factorization's, then one for right-hand-side blocks of each width
+  // (rhs_width), so that no call changes what another launch of this handle, captured ones included, reads
   Problem *dprob = nullptr;
   void *dA = nullptr, *dT = nullptr, *dBw = nullptr;
   size_t bw_cap = 0;
@@ -421,10 +423,20 @@ struct hqr_factors {
 
 namespace {
 
-int run_graph(hqr_factors *F, DevGraph &g, cudaStream_t s) {
+// Right-hand-side block widths of rhs_width; on the device F->dprob[1 + i] has width kRhsWidths[i].
+constexpr int kRhsWidths[3] = {4, 8, 16};
+
+// Runs a task graph of F; wb: right-hand-side block width of an apply graph, 0 for the factorization.
+int run_graph(hqr_factors *F, DevGraph &g, cudaStream_t s, int wb = 0) {
+  Problem prob = F->prob;
   EngineParams p{};
-  p.tc = F->prob.tc;
+  p.tc = prob.tc;
   p.probs = F->dprob;
+  for (int i = 0; i < 3; ++i)
+    if (wb == kRhsWidths[i]) {
+      prob.wb = wb;
+      p.probs = F->dprob + 1 + i;
+    }
   p.tasks = g.tasks;
   p.ntasks = g.ntasks;
   p.succ = g.succ;
@@ -433,7 +445,7 @@ int run_graph(hqr_factors *F, DevGraph &g, cudaStream_t s) {
   p.ctl = g.ctl;
   p.timeout_ns = g_timeout_ns;
   p.trace = (F->dtrace && F->trace_cap >= (size_t)g.ntasks) ? F->dtrace : nullptr;
-  const size_t smem = smem_for(F->prec, F->prob);
+  const size_t smem = smem_for(F->prec, prob);
   CK(g.reset(s));
   if (!F->ev0) {
     CK(cudaEventCreate(&F->ev0));
@@ -482,8 +494,10 @@ int push_problem(hqr_factors *F) {
   F->prob.A = F->dA;
   F->prob.T = F->dT;
   F->prob.B = F->dBw;
-  if (!F->dprob) CK(cudaMalloc(&F->dprob, sizeof(Problem)));
-  CK(cudaMemcpy(F->dprob, &F->prob, sizeof(Problem), cudaMemcpyHostToDevice));
+  Problem v[4] = {F->prob, F->prob, F->prob, F->prob};
+  for (int i = 0; i < 3; ++i) v[1 + i].wb = kRhsWidths[i];
+  if (!F->dprob) CK(cudaMalloc(&F->dprob, sizeof(v)));
+  CK(cudaMemcpy(F->dprob, v, sizeof(v), cudaMemcpyHostToDevice));
   return setup_done();
 }
 
@@ -820,16 +834,13 @@ int hqr_apply_q(hqr_factors *F, int trans, void *dB, int ldb, int nrhs, void *st
   const int nslab = (nrhs + wa - 1) / wa;
   const size_t need = (size_t)F->Mp * nslab * wa;
   const size_t es = elem_size(F->prec);
-  if (need > F->bw_cap || wa != F->prob.wb) {
+  if (need > F->bw_cap) {
     CK(cudaStreamSynchronize(s));
-    if (need > F->bw_cap) {
-      cudaFree(F->dBw);
-      F->dBw = nullptr;
-      F->bw_cap = 0;
-      if (!cuda_ok(cudaMalloc(&F->dBw, es * need), "cudaMalloc(B)")) return HQR_ERR_NOMEM;
-      F->bw_cap = need;
-    }
-    F->prob.wb = wa;
+    cudaFree(F->dBw);
+    F->dBw = nullptr;
+    F->bw_cap = 0;
+    if (!cuda_ok(cudaMalloc(&F->dBw, es * need), "cudaMalloc(B)")) return HQR_ERR_NOMEM;
+    F->bw_cap = need;
     int st = push_problem(F);
     if (st) return st;
   }
@@ -854,7 +865,7 @@ int hqr_apply_q(hqr_factors *F, int trans, void *dB, int ldb, int nrhs, void *st
                                                     F->nb, wa, total);
   CK(cudaGetLastError());
   g_launches += 1;
-  int st = run_graph(F, it->second, s);
+  int st = run_graph(F, it->second, s, wa);
   if (st) return st;
   const long long tot2 = (long long)F->M * nrhs;
   if (F->prec == HQR_FP64)

@@ -377,3 +377,27 @@ def test_apply_q_block_widths(dtype):
             out = F.apply_q(Bd if dtype == "f64" else Bd.float(), trans=trans).double().cpu().numpy()
             err = np.max(np.abs(out - o_apply_q(Fo, B, trans=trans)))
             assert err <= (1e-12 if dtype == "f64" else 5e-6) * np.linalg.norm(B), (k, trans)
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_captured_refactor_between_block_widths(dtype):
+    """A factorization captured in a CUDA graph gives the same bits when replayed
+    after right-hand sides of another block width than those before the capture."""
+    nb, ib, m, n = 64, 16, 12, 2
+    td = torch.float64 if dtype == "f64" else torch.float32
+    A = [torch.from_numpy(inputs.gaussian(m * nb, n * nb, seed=230 + q)).cuda().to(td).t().contiguous().t()
+         for q in range(2)]
+    F = hqr.geqrf(A[0], nb, ib, hqr_elim_list(m, n, 4, 1, GREEDY, GREEDY))
+    ref = F.tiles().clone()
+    F.apply_q(torch.ones(m * nb, 3, dtype=td, device="cuda"), trans=True)  # blocks of 4
+    s = torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=s):
+        F.refactor_async(A[0], s)
+    F.refactor(A[1])
+    F.apply_q(torch.ones(m * nb, 2000, dtype=td, device="cuda"), trans=True)  # blocks of 16
+    g.replay()
+    torch.cuda.synchronize()
+    assert F.status() == 0
+    assert torch.equal(F.tiles(), ref)
