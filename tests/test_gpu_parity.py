@@ -328,6 +328,28 @@ def test_panel_scaled_columns(shape, a, nb, ib, dtype):
     assert np.max(err) <= (R_TOL if dtype == "f64" else 5e-6)
 
 
+@pytest.mark.parametrize("shape,a,nb,ib", [((1, 1), 1, 64, 16), ((2, 1), 2, 64, 16), ((2, 1), 1, 64, 16), ((2, 1), 2, 128, 32),
+                                           ((3, 2), 2, 16, 8)])
+@pytest.mark.parametrize("dtype,exps", [("f32", (13, 116)), ("f32", (10, 119)), ("f32", (6, 121)), ("f32", (-23, -116)),
+                                        ("f32", (-20, -120)), ("f32", (120, -120, 0)), ("f64", (60, 965)), ("f64", (60, 980)),
+                                        ("f64", (-60, -1000)), ("f64", (1000, -1000, 0))])
+def test_panel_columns_of_far_sizes(shape, a, nb, ib, dtype, exps):
+    """GEQRT, TSQRT and TTQRT blocks whose columns are of ordinary size next to
+    columns near the type's largest or smallest numbers: R must be the unscaled
+    R with scaled columns (a column scaling by powers of two commutes with QR),
+    each column within R_TOL (FP32: 5e-6) of its own norm."""
+    m, n = shape
+    A = inputs.gaussian(m * nb, n * nb, seed=270 + nb + a)
+    recs = hqr_elim_list(m, n, a, 1, FLAT, FLAT)
+    scale = np.ldexp(1.0, np.resize(exps, n * nb))
+    A = A.astype(np.float32).astype(np.float64) if dtype == "f32" else A
+    base = tile_qr(A, nb, ib, recs).R()
+    As = torch.from_numpy(A * scale).cuda()
+    R = hqr.geqrf(As if dtype == "f64" else As.float(), nb, ib, recs).R().double().cpu().numpy()
+    err = np.abs(R / scale - base) / np.linalg.norm(A, axis=0)
+    assert np.max(err) <= (R_TOL if dtype == "f64" else 5e-6)
+
+
 @pytest.mark.parametrize("dtype,nb,ib,w", [("f64", 64, 32, 16), ("f64", 88, 8, 16), ("f64", 96, 16, 8), ("f64", 96, 16, 16),
                                            ("f64", 104, 8, 4), ("f64", 40, 4, 4), ("f32", 128, 16, 16), ("f32", 128, 16, 12),
                                            ("f32", 128, 32, 16), ("f32", 64, 8, 64), ("f32", 136, 8, 8)])
