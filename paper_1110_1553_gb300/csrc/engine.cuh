@@ -726,10 +726,14 @@ __device__ __forceinline__ void form_reflector(int mode, Real *P, int ld, int L,
   } else {
     const int r0 = refl_begin(mode, j), r1 = refl_end(mode, j, L, q0);
     Real am = 0;
-    for (int k = r0 + lane; k < r1; k += 32) am = fmax(am, fabs(col[k]));
+    unsigned any = 0;  // not a zero column (am does not see NaN)
+    for (int k = r0 + lane; k < r1; k += 32) {
+      am = fmax(am, fabs(col[k]));
+      any |= magnitude_key(col[k]);
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) am = fmax(am, __shfl_xor_sync(0xffffffffu, am, o));
-    if (am != Real(0)) {
+    if (__any_sync(0xffffffffu, any != 0)) {
       const Real inv = Real(1) / am;
       Real s2 = 0;
       for (int k = r0 + lane; k < r1; k += 32) {

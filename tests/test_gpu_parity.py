@@ -350,6 +350,31 @@ def test_panel_columns_of_far_sizes(shape, a, nb, ib, dtype, exps):
     assert np.max(err) <= (R_TOL if dtype == "f64" else 5e-6)
 
 
+@pytest.mark.parametrize("shape,a", [((1, 1), 1), ((2, 1), 2), ((2, 1), 1)])
+@pytest.mark.parametrize("prec,nb,ib", [("f64", 32, 8), ("f64", 64, 16), ("f32", 32, 8), ("f32", 128, 16), ("tensor", 128, 128)])
+@pytest.mark.parametrize("dense", [False, True])
+def test_nan_reaches_r(shape, a, prec, nb, ib, dense):
+    """One NaN below the diagonal, in column c of the last tile, among zeros or
+    in a full tile (where the reflectors before c spread it over the column,
+    so that nothing else is left there): R(c, c) is NaN, and the columns before
+    c are what they are without it."""
+    m, n = shape
+    A = inputs.gaussian(m * nb, nb, seed=290 + nb)
+    row = m * nb - 2 if m == 1 or a == 2 else nb
+    if not dense:
+        A[(m - 1) * nb + 1:] = 0
+        A[(m - 1) * nb] = 0 if m > 1 else A[0]
+    recs = hqr_elim_list(m, 1, a, 1, FLAT, FLAT)
+    dt = torch.float64 if prec == "f64" else torch.float32
+    for c in (0, 1, ib - 1, nb // 2, nb - 3):
+        B = torch.from_numpy(A.copy()).to(dt)
+        R0 = hqr.geqrf(B.cuda(), nb, ib, recs, tensor=prec == "tensor").R().cpu()
+        B[row, c] = float("nan")
+        R = hqr.geqrf(B.cuda(), nb, ib, recs, tensor=prec == "tensor").R().cpu()
+        assert torch.isnan(R[c, c]), c
+        assert torch.equal(R[:, :c], R0[:, :c]), c
+
+
 @pytest.mark.parametrize("dtype,nb,ib,w", [("f64", 64, 32, 16), ("f64", 88, 8, 16), ("f64", 96, 16, 8), ("f64", 96, 16, 16),
                                            ("f64", 104, 8, 4), ("f64", 40, 4, 4), ("f32", 128, 16, 16), ("f32", 128, 16, 12),
                                            ("f32", 128, 32, 16), ("f32", 64, 8, 64), ("f32", 136, 8, 8)])
