@@ -14,6 +14,7 @@
 #include "../../include/hqr.h"
 #include "engine.cuh"
 #include "hqr_internal.h"
+#include "smem_limits.h"
 
 using namespace hqr;
 
@@ -246,15 +247,16 @@ size_t smem_for(int prec, const Problem &P) {
 
 // CTAs for a launch: every SM filled to the occupancy the kernel allows.
 int ctas_for(int prec, bool tc, size_t smem, int ntasks, int *grid) {
-  static size_t attr[3] = {0, 0, 0};
+  static SmemLimits<3> limits;
   const void *k = sched_kernel(prec, tc);
   const int slot = prec == HQR_FP64 ? 0 : (tc ? 2 : 1);
-  if (attr[slot] < smem) {
-    CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr[slot] = smem;
-  }
   int dev = 0, sms = 0, per_sm = 0;
   CK(cudaGetDevice(&dev));
+  if (!limits.raise(dev, slot, smem, [&] {
+        return cuda_ok(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                       "cudaFuncSetAttribute(shared memory)");
+      }))
+    return HQR_ERR_CUDA;
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NT, smem));
   if (per_sm < 1) {

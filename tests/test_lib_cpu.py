@@ -103,3 +103,48 @@ def test_validator_agrees_with_oracle_on_mutations(lib):
     for name, M in _mutations(L):
         assert validate(M, 16, 4) is not None
         assert hqr.validate_list(16, 4, M) == hqr.ERR_INVALID_LIST, name
+
+
+SMEM_LIMITS = r"""
+#include "smem_limits.h"
+#include <cstdio>
+#include <thread>
+#include <vector>
+using namespace hqr;
+static size_t attr[3][2];  // what a device's kernel was set to: 2 devices in the record, one beyond
+static int calls;
+int main() {
+  SmemLimits<2, 2> rec;
+  auto raise = [&](int dev, int k, size_t b) { return rec.raise(dev, k, b, [&] { ++calls; attr[dev][k] = b; return true; }); };
+  // every launch on every device finds at least its bytes, and no limit is lowered
+  const size_t seq[][3] = {{0, 0, 90}, {1, 0, 60}, {0, 0, 70}, {0, 1, 50}, {1, 1, 50}, {1, 0, 95}, {0, 0, 90}, {2, 0, 40}, {2, 0, 30}};
+  for (auto &q : seq) {
+    const size_t before = attr[q[0]][q[1]];
+    if (!raise((int)q[0], (int)q[1], q[2]) || attr[q[0]][q[1]] < q[2]) return 1;
+    if (q[0] < 2 && attr[q[0]][q[1]] < before) return 2;
+  }
+  if (calls != 7) return 3;
+  // a failed set is reported and tried again
+  if (rec.raise(0, 1, 80, [] { return false; }) || !raise(0, 1, 80) || attr[0][1] != 80) return 4;
+  // two threads: the largest value stays
+  std::vector<std::thread> t;
+  for (int i = 0; i < 8; ++i) t.emplace_back([&, i] { for (int b = 100 + i; b < 4000; b += 8) raise(0, 0, (size_t)b); });
+  for (auto &x : t) x.join();
+  return attr[0][0] == 3999 ? 0 : 5;
+}
+"""
+
+
+def test_shared_memory_limits_per_device(tmp_path):
+    """The record behind the scheduler launches, on a fake of the attribute: a
+    limit that one device was granted says nothing about another device."""
+    import shutil
+    import subprocess
+    gxx = shutil.which("g++")
+    if gxx is None:
+        pytest.skip("no g++")
+    src, exe = tmp_path / "limits.cpp", tmp_path / "limits"
+    src.write_text(SMEM_LIMITS)
+    subprocess.run([gxx, "-std=c++17", "-O1", "-pthread", "-I", os.path.join(ROOT, "paper_1110_1553_gb300", "csrc"), str(src),
+                    "-o", str(exe)], check=True)
+    assert subprocess.run([str(exe)]).returncode == 0
