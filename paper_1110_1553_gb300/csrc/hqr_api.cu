@@ -337,16 +337,23 @@ void drop_t32(int prec, Problem &P) {
 // `tiles`: tiles of the factorization; 0 for plans and server requests, whose
 // launches hold other problems too and whose results must not depend on them
 // (the order of sums follows the width).
-// FP64 (ms, slabs of 16 / 8 / 4): 8 x 8 tiles of 64 2.49 / 2.15 / 1.98, 8 x 2
-// of 128 2.40 / 1.94 / 1.83, 16 x 16 of 64 5.7 / 4.9 / 4.6 (4 doubles the tasks
-// the host builds), 63 x 8 of 64 4.3 / 4.0 / 4.9; inner blocks of 32 (more
-// arithmetic per staged block): 16 x 16 of 128 27.8 / 23.9 / 24.7, 32 x 16 of 128
-// 47 / 40 / 50, 128 x 8 of 256 259.5 / 255.5 (and 66 ms more on the host, so it
-// stays at 16). FP32 on CUDA cores (slabs of 64 / 32 / 16): 20 x 14 of 128 22.5 /
-// 17.7 / 10.1 and 64 x 4 of 128 4.8 / 3.8 / 2.4 (slabs no wider than a block also
-// let the panels split, see split_ib_for), 10 x 5 of 64 1.29 / 1.04 / 0.93, 128 x
-// 8 of 64 3.10 / 2.48 / 2.54, 32 x 32 of 128 47 / 46 / 29, 128 x 16 of 128 29.8 /
-// 29.2 / 35.7, 160 uneven problems 19.6 / 21.1 / 27.7.
+// The limits weigh a kept factorization (first figure, ms) against a one-shot
+// call, which builds the graph too (in brackets). FP64, slabs of 16 / 8 / 4:
+//  blocks of 16, up to 2^20 elements: 8 x 8 tiles of 64 2.46 (2.9) / 2.19 (2.9) /
+//   2.01 (3.5), 8 x 8 of 128 7.5 (8.3) / 6.3 (8.1) / 6.3 (11); above: 32 x 4 of 96
+//   3.6 (4.6) / 3.1 (5.1) / 2.8 (7.4), 32 x 4 of 128 5.7 (7.0) / 4.8 (7.9) / 5.3 (13), 32 x
+//   4 of 256 23 (28) / 20 (31) / 29 (64); 17 x 8 of 64 3.2 (4.0) / 2.7 (4.3) / 2.5 (6.2)
+//  up to 320 tiles and, with blocks of 16, 10 x 2^20 elements: 40 x 8 of 64 3.8 (5.5) /
+//   3.4 (7.1) / 3.4 (12), 16 x 16 of 128 19 (23) / 16 (27) / 21 (54); above: 41 x 8 of 64
+//   3.8 (5.6) / 3.5 (7.1) / 3.5 (13), 63 x 8 of 64 4.3 (7.0) / 4.1 (9.7) / 4.9 (19), 16 x 16
+//   of 256 98 (112) / 93 (133) / 143 (311)
+//  blocks of 32, up to 320 tiles: 64 x 4 of 128 8.0 (10) / 7.0 (12) / 9.0 (21), 16 x 16 of
+//   192 52 (58) / 43 (61) / 64 (127); above: 40 x 12 of 128 26 (34) / 26 (44) / 37 (92)
+//  blocks of 8: 16 x 16 of 256 128 (143) / 102 (154) / 163 (357).
+// FP32 on CUDA cores, slabs of 64 (tiles of 256: 32) / 16; slabs no wider than a
+// block also let the panels split, see split_ib_for: 8 x 8 of 64 1.24 (1.5) / 1.19
+// (1.6), 40 x 20 of 128 13.5 (16) / 10.1 (30), 24 x 24 of 192 27 (30) / 20 (46); above 600
+// tiles of more than 128: 40 x 20 of 192 27 (31) / 28 (67), of 256 62 (74) / 54 (122).
 void choose_widths(int prec, int nb, int ib, Problem &P, long long tiles = 0) {
   P.wb = std::min(16, nb);
   P.tc = use_tc(prec, nb) ? 1 : 0;
@@ -358,15 +365,17 @@ void choose_widths(int prec, int nb, int ib, Problem &P, long long tiles = 0) {
     P.vc = 16;
     return;
   }
+  const long long area = tiles * nb * nb;  // elements
   if (prec == HQR_FP64) {
     P.w = std::min(16, nb);
-    if (tiles > 0 && nb >= 16) P.w = tiles <= 128 && ib <= 16 ? 4 : (tiles <= (nb >= 128 && ib > 16 ? 512 : 320) ? 8 : 16);
+    if (tiles > 0 && nb >= 16)
+      P.w = tiles <= 128 && ib <= 16 && area <= 1 << 20 ? 4 : (tiles <= 320 && (ib > 16 || ib <= 8 || area <= 10 << 20) ? 8 : 16);
     P.wt = nb > 128 ? 8 : std::min(16, nb);
     P.vc = nb > 128 ? std::min(ib, 8) : std::min(ib, 16);
   } else {
     P.w = nb >= 256 ? 32 : std::min(64, nb);
     // (fewer than 12 tiles keep whole panels)
-    if (tiles >= 12 && tiles <= 1024 && ib <= 16 && nb >= 16) P.w = 16;
+    if (tiles >= 12 && tiles <= (nb > 128 ? 600 : 1024) && ib <= 16 && nb >= 16) P.w = 16;
     P.wt = nb >= 256 ? 16 : std::min(32, nb);
     P.vc = std::min(ib, 16);
   }

@@ -496,3 +496,18 @@ def test_fused_solve_steps_lead_their_predecessors_successors(kind):
             assert lst[0] == r, (op, int(q), int(r), [int(x) for x in lst[:4]])
             checked += 1
     assert checked >= 2 * 3 * (n - 2)  # every round's two chains
+
+
+@pytest.mark.parametrize("prec,m,n,nb,ib,width", [
+    ("f64", 8, 8, 64, 16, 4), ("f64", 16, 8, 64, 16, 4), ("f64", 8, 8, 128, 16, 4), ("f64", 16, 4, 256, 8, 8), ("f64", 17, 8, 64, 16, 8),
+    ("f64", 32, 4, 96, 16, 8), ("f64", 32, 4, 256, 16, 8), ("f64", 16, 11, 256, 16, 16), ("f64", 16, 11, 256, 8, 8),
+    ("f64", 16, 16, 128, 32, 8), ("f64", 40, 8, 64, 16, 8), ("f64", 41, 8, 64, 16, 16), ("f64", 41, 8, 128, 32, 16), ("f64", 2, 2, 8, 4, 8),
+    ("f32", 11, 1, 64, 16, 64), ("f32", 12, 2, 64, 16, 16), ("f32", 32, 32, 128, 16, 16), ("f32", 50, 12, 192, 16, 16),
+    ("f32", 43, 14, 192, 16, 64)])
+def test_slab_widths_by_size(prec, m, n, nb, ib, width):
+    """Columns of a factorization's update tasks on both sides of the limits that
+    keep narrow slabs to graphs the host builds in less time than they save."""
+    p = hqr.FP64 if prec == "f64" else hqr.FP32
+    tasks, _, _ = hqr.task_graph(m, n, nb, ib, hqr_elim_list(m, n, 4, 1, GREEDY, GREEDY), prec=p)
+    cw = tasks[np.isin(tasks[:, 0], [UNMQR, TSMQR, TTMQR]) & (tasks[:, 1] == 0)][:, 7]
+    assert len(cw) == 0 or cw.max() == width
