@@ -694,9 +694,13 @@ __device__ __forceinline__ bool in_plain_range(float alpha, float ss) {
 // and scale w far from the type's limits, where products of all sizes gave
 // NaN (FP32 columns of 1e4 beside 1e35) or few bits (1e-6 beside 1e-36).
 template <typename Real>
+struct Safe {  // of the type's (FP64: its high word's) bits: mantissa, exponent bias, and the range above
+  static constexpr int mant = sizeof(Real) == 8 ? 20 : 23, bias = sizeof(Real) == 8 ? 1023 : 127, edge = sizeof(Real) == 8 ? 400 : 60;
+};
+template <typename Real>
 __device__ __forceinline__ int column_shift(unsigned key) {
-  constexpr int mant = sizeof(Real) == 8 ? 20 : 23, bias = sizeof(Real) == 8 ? 1023 : 127, edge = sizeof(Real) == 8 ? 400 : 60;
-  const int e = (int)(key >> mant) - bias;  // 2^e <= |a| < 2^(e + 1); bias + 1: not finite
+  constexpr int bias = Safe<Real>::bias, edge = Safe<Real>::edge;
+  const int e = (int)(key >> Safe<Real>::mant) - bias;  // 2^e <= |a| < 2^(e + 1); bias + 1: not finite
   if (key == 0 || e == bias + 1) return 0;
   return e > edge ? edge - e : (e < -edge ? -edge - e : 0);
 }
@@ -757,34 +761,47 @@ __device__ __forceinline__ void form_reflector(int mode, Real *P, int ld, int L,
   }
 }
 
-// Shift of column c of a block by the eight lanes of its group: pc[0 .. np) and
-// rc[0 .. nr), its parts in the killed tile (GE: the tile itself) and in R. The
-// first column needs none: it is no other reflector's operand. The check costs
-// 512^2 FP64 QR + Q 0.7 % (2.648 -> 2.667 ms), a 130 x 70 R 1.2 %, the FP32 fit
-// of 2500 x 1700 0.7 %, mostly as code that every block runs through: with
-// scale_column inlined as well 1.6 %, 2 % and 1.4 %.
+// The column that this lane's group of eight found to be of extreme size. The
+// first column needs no shift: it is no other reflector's operand.
 template <typename Real>
-__device__ __forceinline__ void measure_column(const Real *pc, int np, const Real *rc, int nr, int c, Shared<Real> &sh) {
-  const int part = threadIdx.x & 7, lane = threadIdx.x & 31;
-  unsigned m = 0;
-#pragma unroll 4
-  for (int k = part; k < np; k += 8) m = max(m, magnitude_key(pc[k]));
-  for (int k = part; k < nr; k += 8) m = max(m, magnitude_key(rc[k]));
-#pragma unroll
-  for (int o = 4; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffu << (lane & 24), m, o));
-  const int e = c == 0 ? 0 : column_shift<Real>(m);
-  if (part == 0) {
+__device__ __noinline__ void flag_column(unsigned key, int c, Shared<Real> &sh) {
+  const int e = c == 0 ? 0 : column_shift<Real>(key);
+  if ((threadIdx.x & 7) == 0 && e != 0) {
     sh.shift[c] = e;
-    if (e != 0) sh.extreme = sh.redo = 1;
+    sh.extreme = sh.redo = 1;
   }
 }
 
-// pc[0 .. np) and rc[0 .. nr) times 2^e.
+// Looks at the size of column c by the eight lanes of its group: pc[0 .. np) and
+// rc[0 .. nr), its parts in the killed tile (GE: the tile itself) and in R. Every
+// block runs through this once and pays for its instructions more than for
+// its loads: with the shift found here, two loops and the scaling inlined
+// 512^2 FP64 QR + Q took 2.70 ms, so 2.67, without a check 2.65; FP32 2500 x 1700
+// 13.6, 13.45 and 13.4; FP32 with blocks of 8 loses most, 3 to 4 %.
 template <typename Real>
-__device__ __noinline__ void scale_column(Real *pc, int np, Real *rc, int nr, int e) {
-  const int part = threadIdx.x & 7;
-  for (int k = part; k < np; k += 8) pc[k] = times_pow2(pc[k], e);
-  for (int k = part; k < nr; k += 8) rc[k] = times_pow2(rc[k], e);
+__device__ __forceinline__ void look_at_column(const Real *pc, int np, const Real *rc, int nr, int c, Shared<Real> &sh) {
+  const int lane = threadIdx.x & 31;
+  unsigned m = 0;
+#pragma unroll 4
+  for (int k = lane & 7; k < np + nr; k += 8) m = max(m, magnitude_key(k < np ? pc[k] : rc[k - np]));
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffu << (lane & 24), m, o));
+  constexpr unsigned lo = (unsigned)(Safe<Real>::bias - Safe<Real>::edge) << Safe<Real>::mant,
+                     hi = (unsigned)(Safe<Real>::bias + Safe<Real>::edge + 1) << Safe<Real>::mant;
+  if (m - lo >= hi - lo && m != 0) flag_column(m, c, sh);
+}
+
+// Every column of the block times 2^shift, or (back) its rows of R times 2^-shift.
+template <typename Real>
+__device__ __noinline__ void scale_columns(int mode, Real *P, int ld, int L, int ib, Real *Rt, int ldt, int q0, bool back,
+                                           const Shared<Real> &sh) {
+  const int part = threadIdx.x & 7, c = (int)threadIdx.x >> 3;
+  if (c >= ib || sh.shift[c] == 0) return;
+  const int e = back ? -sh.shift[c] : sh.shift[c];
+  Real *pc = P + (size_t)c * ld, *rc = mode == PANEL_GE ? pc : Rt + (size_t)c * ldt;
+  for (int k = part; k <= c; k += 8) rc[k] = times_pow2(rc[k], e);
+  if (!back)
+    for (int k = (mode == PANEL_GE ? c + 1 : 0) + part, k1 = refl_end(mode, c, L, q0); k < k1; k += 8) pc[k] = times_pow2(pc[k], e);
 }
 
 // Householder factorization of one block of ib columns held in shared memory,
@@ -817,7 +834,7 @@ __device__ void factor_block(int mode, Real *P, int ld, int L, int ib, Real *Rt,
   const int grp = warp - first;
   const int part = lane & (LPC - 1), c = grp * CPW + lane / LPC;
   const bool colw = grp >= 0 && grp * CPW < ib, has = colw && c < ib;
-  Real *pc = P + (size_t)(has ? c : 0) * ld, *rtc = Rt + (size_t)(has ? c : 0) * ldt;
+  Real *pc = P + (size_t)(has ? c : 0) * ld;
   Real s = 0;  // x_j^T a_c (every lane of the column's group)
   auto products = [&](int j) {  // column j with this group's column
     const Real *col = P + (size_t)j * ld;
@@ -851,6 +868,7 @@ __device__ void factor_block(int mode, Real *P, int ld, int L, int ib, Real *Rt,
     const Real tau = sh.tau[j];
     Tq[lane + (size_t)j * ldq] = lane < j ? -tau * y : (lane == j ? tau : Real(0));
   };
+  if (tid < IBMAX) sh.shift[tid] = 0;
   if (tid == 0) sh.redo = sh.extreme = 0;
   __syncthreads();
   for (int j = 0; j < ib; ++j) {
@@ -883,20 +901,21 @@ __device__ void factor_block(int mode, Real *P, int ld, int L, int ib, Real *Rt,
     if (warp == 1 && j > 1) t_column(j - 2);
     if (colw) products(j);
     if (j == 0 && has)  // in the shadow of the first norm
-      measure_column(pc, mode == PANEL_GE ? L : refl_end(mode, c, L, q0), rtc, mode == PANEL_GE ? 0 : c + 1, c, sh);
+      look_at_column(pc, mode == PANEL_GE ? L : refl_end(mode, c, L, q0), Rt + (size_t)c * ldt, mode == PANEL_GE ? 0 : c + 1, c, sh);
     __syncthreads();
     // the column was scaled in place, or columns of extreme size are to be (the same in every thread)
     if (sh.redo == j + 1) {
-      if (j == 0 && sh.extreme && has && sh.shift[c] != 0)
-        scale_column(pc, mode == PANEL_GE ? L : refl_end(mode, c, L, q0), rtc, mode == PANEL_GE ? 0 : c + 1, sh.shift[c]);
+      if (j == 0 && sh.extreme) {
+        scale_columns(mode, P, ld, L, ib, Rt, ldt, q0, false, sh);
+        __syncthreads();
+      }
       if (colw) products(j);
       __syncthreads();
     }
   }
   if (colw) apply(ib - 1, ib);
   __syncthreads();
-  if (sh.extreme && has && sh.shift[c] != 0)  // R back
-    scale_column(mode == PANEL_GE ? pc : rtc, c + 1, rtc, 0, -sh.shift[c]);
+  if (sh.extreme) scale_columns(mode, P, ld, L, ib, Rt, ldt, q0, true, sh);
   if (warp == 1) {
     if (ib > 1) t_column(ib - 2);
     __syncwarp();
