@@ -117,6 +117,7 @@ struct EngineParams {
   long long timeout_ns;
   unsigned long long *trace;  // optional: per task start, end (globaltimer), SM id
   int tc;                     // some problem uses the tensor-core kernels (launch the TC variant)
+  int keep_rhs;               // a CTA keeps a successor of an update of a right-hand side (see hqr_sched)
 };
 
 template <typename Real>
@@ -2213,19 +2214,17 @@ __global__ void __launch_bounds__(NT, TC ? 1 : 2) hqr_sched(EngineParams p) {
   // its successors are released, which cannot end the run early since the
   // counter reaches the task count only when no task has unfinished
   // successors. Seven warps release the successors (a solve step has up to
-  // one per tile of the vector). After a least-squares vector task (or an update
-  // of a right-hand side), the most
-  // critical successor that the release makes ready (successors are listed by
-  // decreasing bottom level) stays with this CTA and runs next without a trip
-  // through the queues: the solve chain pays neither the push nor another
-  // CTA's claim per step (measured: 7.0 -> 4.3 us between steps), and the sum
-  // of a column tile's A^T r partials, then the solve step that needs it, run as
-  // soon as the last partial is done instead of queuing behind the other
-  // columns' partials. After such a task warp 1 claims only if nothing was kept
-  // (after the release), so a kept task never meets a claimed one. The updates
-  // of a right-hand side form such chains too (Q^T of 300 columns on 64 x 8 tiles
-  // of 128: 1.29 -> 1.09 ms). (Keeping after factorization tasks as well cost the
-  // 512^2 FP64 latency case 2 %.)
+  // one per tile of the vector). After a least-squares vector task, or an update
+  // of a right-hand side where keep_rhs says so, the most critical successor
+  // that the release makes ready (successors are listed by decreasing bottom level) stays with
+  // this CTA and runs next without a trip through the queues: the solve chain
+  // pays neither the push nor another CTA's claim per step (measured: 7.0 ->
+  // 4.3 us between steps), and the sum of a column tile's A^T r partials, then the
+  // solve step that needs it, run as soon as the last partial is done instead
+  // of queuing behind the other columns' partials. After such a task warp 1
+  // claims only if nothing was kept (after the release), so a kept task never
+  // meets a claimed one.
+  // Keeping after factorization tasks as well cost the 512^2 FP64 latency case 2 %.
   unsigned pending = 0;
   if (threadIdx.x == 0) {
     sh.kept = -1;
@@ -2241,7 +2240,7 @@ __global__ void __launch_bounds__(NT, TC ? 1 : 2) hqr_sched(EngineParams p) {
     if (tid < 0) break;
     const Task t = p.tasks[tid];
     const Geo<Real> g(p.probs[t.pid]);
-    const bool keeps = t.op >= OP_RESID || t.tgt == 1;
+    const bool keeps = t.op >= OP_RESID || (t.tgt == 1 && p.keep_rhs);
     const uint64_t t_start = (p.trace && threadIdx.x == 0) ? ptx::globaltimer() : 0;
     if (TC && t.op <= OP_TTMQR && p.probs[t.pid].tc) {
       if (!tc_task<Real, TC>(p, g, t, sh, dyn_raw, ts, tph) && threadIdx.x == 0) set_error(p, HQR_ERR_TIMEOUT, tid);

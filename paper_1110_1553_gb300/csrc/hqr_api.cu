@@ -437,11 +437,24 @@ namespace {
 // Right-hand-side block widths of rhs_width; on the device F->dprob[1 + i] has width kRhsWidths[i].
 constexpr int kRhsWidths[3] = {4, 8, 16};
 
-// Runs a task graph of F; wb: right-hand-side block width of an apply graph, 0 for the factorization.
-int run_graph(hqr_factors *F, DevGraph &g, cudaStream_t s, int wb = 0) {
+// Whether a CTA that finishes an update of a right-hand side keeps its most critical successor. The
+// updates of one block form a chain, which gains, but the CTA's next claim then waits for the release:
+// short tasks and few blocks gain, many long FP64 tasks lose. Q^T in ms, kept and not: 300 columns on
+// 64 x 8 tensor-core tiles 1.09 / 1.29, 1500 on 100 x 2 FP32 tiles of 32 0.83 / 1.32, on 32 x 4 of 128 1.67 /
+// 1.58; FP64 1500 on 32 x 4 tiles of 16 0.62 / 0.83, of 32 1.22 / 1.18, of 64 3.5 / 3.2, of 128 12.3 / 11.3, 500 on
+// 100 x 2 of 256 29.3 / 26.4; one block of 4 on 32 x 4 of 64 0.395 / 0.418, of 128 1.29 / 1.32, on 100 x 2 of 96
+// 0.61 / 0.53 (there the rows' chains run side by side); 10 blocks on 32 x 4 of 128 1.72 / 1.64.
+bool keeps_rhs(int prec, int nb, int m, int blocks) {
+  return prec != HQR_FP64 || nb < 64 || (blocks <= 4 && m <= 64);
+}
+
+// Runs a task graph of F; for an apply graph wb: width of the right-hand-side blocks, blocks: their
+// number; 0 for the factorization.
+int run_graph(hqr_factors *F, DevGraph &g, cudaStream_t s, int wb = 0, int blocks = 0) {
   Problem prob = F->prob;
   EngineParams p{};
   p.tc = prob.tc;
+  p.keep_rhs = keeps_rhs(F->prec, F->nb, F->m, blocks);
   p.probs = F->dprob;
   for (int i = 0; i < 3; ++i)
     if (wb == kRhsWidths[i]) {
@@ -876,7 +889,7 @@ int hqr_apply_q(hqr_factors *F, int trans, void *dB, int ldb, int nrhs, void *st
                                                     F->nb, wa, total);
   CK(cudaGetLastError());
   g_launches += 1;
-  int st = run_graph(F, it->second, s, wa);
+  int st = run_graph(F, it->second, s, wa, nslab);
   if (st) return st;
   const long long tot2 = (long long)F->M * nrhs;
   if (F->prec == HQR_FP64)
@@ -1179,6 +1192,7 @@ int plan_enqueue(hqr_ls_plan *P, cudaStream_t s, bool timed) {
   auto params = [&](const DevGraph &g, int tc, unsigned long long *trace) {
     EngineParams p{};
     p.tc = tc;
+    p.keep_rhs = 1;  // one right-hand side per problem
     p.probs = P->dprobs;
     p.tasks = g.tasks;
     p.ntasks = g.ntasks;
