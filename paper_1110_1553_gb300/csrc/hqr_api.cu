@@ -385,15 +385,23 @@ void choose_widths(int prec, int nb, int ib, Problem &P, long long tiles = 0) {
 }
 
 // Columns of a right-hand-side block (one task of Q or Q^T on CUDA cores): the
-// replay is a chain of updates, so few row tiles and columns take narrow, short
-// tasks, many of them the cheaper wide ones. Times of Q in ms at 4 / 8 / 16
-// columns: FP64 8 tiles of 64, 512 columns 0.51 / 0.61 / 1.01, 2000 columns 1.71
-// / 1.31 / 1.31; 32 tiles of 128, 40 columns 2.5 / 2.9 / 4.8, 512 columns 12.2 /
-// 8.0 / 8.1; FP32 20 tiles of 128, 150 columns 0.72 / 0.74 / 0.97, 512 columns
-// 1.85 / 1.11 / 1.03.
+// replay is a chain of updates, so few row tiles times columns take narrow,
+// short tasks, many of them the cheaper wide ones. Q^T in ms at 4 / 8 / 16
+// columns, row tiles x columns on both sides of the limits:
+//  FP64, 4 up to 4096: 8 x 500 (tiles of 64) 0.30 / 0.34 / 0.51, 100 x 40 0.44 / 0.50 / 0.75;
+//   above, where tile sizes differ: 32 x 130 of 32 0.40 / 0.34 / 0.40, of 64 0.60 / 0.66 / 0.98, of
+//   128 2.15 / 2.09 / 3.1; 32 x 250 of 64 0.95 / 0.81 / 1.06, of 128 3.5 / 2.6 / 3.4
+//  FP64, 8 up to 16000: 8 x 1500 0.64 / 0.51 / 0.59, 100 x 130 0.87 / 0.75 / 0.88; equal from 32 x
+//   500 (1.32 / 1.33; of 128 4.5 / 4.4) to 100 x 250 (1.18 / 1.17); above: 32 x 1500 3.6 / 3.2
+//  FP32, 4 up to 2500: 8 x 250 (of 128) 0.20 / 0.22 / 0.28, 100 x 16 0.32 / 0.35 / 0.42; above: 2 x
+//   1500 0.15 / 0.12 / 0.13, of 256 0.40 / 0.26 / 0.29, 100 x 40 0.38 / 0.35 / 0.46, 8 x 500 0.25 /
+//   0.22 / 0.28
+//  FP32, 8 up to 6000: 32 x 130 0.50 / 0.44 / 0.54, of 256 1.9 / 1.5 / 1.7; above: 32 x 250 0.81 /
+//   0.56 / 0.56, of 64 0.49 / 0.34 / 0.32, of 256 3.1 / 2.0 / 1.8.
 int rhs_width(int prec, bool tc, int nb, int m, int nrhs) {
   const long long work = (long long)m * nrhs;
-  const int w = tc ? 16 : (work <= 4096 ? 4 : (work <= (prec == HQR_FP64 ? 16000 : 8192) ? 8 : 16));
+  const bool f64 = prec == HQR_FP64;
+  const int w = tc ? 16 : (work <= (f64 ? 4096 : 2500) ? 4 : (work <= (f64 ? 16000 : 6000) ? 8 : 16));
   return std::min(w, nb);
 }
 

@@ -417,7 +417,7 @@ def test_apply_q_block_widths(dtype):
     Fo = tile_qr(A, nb, ib, recs)
     Ad = torch.from_numpy(A).cuda()
     F = hqr.geqrf(Ad if dtype == "f64" else Ad.float(), nb, ib, recs)
-    for k in (3, 110, 450, 102, 103, 5, 401):
+    for k in (3, 110, 450, 102, 103, 5, 401, 62, 63, 150, 151, 400):
         B = inputs.gaussian(m * nb, k, seed=191 + k).astype(np.float32).astype(np.float64)
         for trans in (True, False):
             Bd = torch.from_numpy(B.copy()).cuda()
