@@ -603,7 +603,8 @@ int hqr_set_slab_widths(int w, int wt, int vc);
  * least two ib blocks per tile) run as one task per ib block plus the
  * updates of the panel's own trailing columns with that block, so that a
  * panel's trailing work spreads over several CTAs. 0 keeps whole panel tasks
- * everywhere; default 64. Returns -1 for min_nb < 0. */
+ * everywhere. Until the first call: 64, and FP64 tiles of 48 with blocks of
+ * 16. Returns -1 for min_nb < 0. */
 int hqr_set_panel_split(int min_nb);
 
 /* hqr_set_split_launch -- least-squares plans created afterwards that hold

@@ -291,8 +291,9 @@ int launch_sched(int prec, const EngineParams &p, size_t smem, cudaStream_t s, i
 int g_w_override = 0, g_wt_override = 0, g_vc_override = 0;
 // Priority policy of task graphs (hqr_set_priority_policy).
 int g_priority_policy = 1;
-// CUDA-core panels of tiles with nb >= this are split into block tasks (hqr_set_panel_split; 0: never).
-int g_split_min_nb = 64;
+// CUDA-core panels of tiles with nb >= this are split into block tasks (hqr_set_panel_split; 0: never,
+// -1: the built-in choice, see split_ib_for).
+int g_split_min_nb = -1;
 // Plans with tensor-core and CUDA-core problems launch them side by side (hqr_set_split_launch).
 int g_split_launch = 1;
 
@@ -300,9 +301,15 @@ int g_split_launch = 1;
 // kernels keep whole panels (one block per tile). FP32 panels on CUDA cores are cheap next to
 // their updates: they are split only where a block spans whole update slabs (measured: splitting
 // blocks narrower than the 64-column FP32 slabs cost 1024 uneven problems 5 %); FP64 panels are
-// split at any slab width (512^2 FP64 QR + Q: -25 % latency).
+// split at any slab width (512^2 FP64 QR + Q: -25 % latency). Built-in: tiles of 64 and more, and the
+// FP64 tiles of 48 that the default configuration takes for 65 to 96 and 129 to 144 columns: a plan of
+// 2000 x 90 takes 1.34 ms with whole panels, 0.94 split (tiles of 64, split: 1.18), 30000 x 144 3.28, 3.19
+// (4.12), 48 uneven problems the same; blocks of 8 and other tiles below 64 lose with many tiles (64 x 8
+// of 48, blocks of 8: 4.4 whole, 5.4 split), as does a single tile (0.135, 0.147).
 int split_ib_for(int prec, const Problem &P) {
-  if (P.tc || g_split_min_nb <= 0 || P.nb < g_split_min_nb) return 0;
+  const bool tiles48 = prec == HQR_FP64 && P.nb == 48 && P.ib == 16 && P.m > 1;
+  const int min_nb = g_split_min_nb >= 0 ? g_split_min_nb : (tiles48 ? 48 : 64);
+  if (P.tc || min_nb == 0 || P.nb < min_nb) return 0;
   if (P.w <= 0 || P.nb / P.ib < 2) return 0;
   if (prec != HQR_FP64 && P.ib % P.w != 0) return 0;
   return P.ib;

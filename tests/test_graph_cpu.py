@@ -511,3 +511,25 @@ def test_slab_widths_by_size(prec, m, n, nb, ib, width):
     tasks, _, _ = hqr.task_graph(m, n, nb, ib, hqr_elim_list(m, n, 4, 1, GREEDY, GREEDY), prec=p)
     cw = tasks[np.isin(tasks[:, 0], [UNMQR, TSMQR, TTMQR]) & (tasks[:, 1] == 0)][:, 7]
     assert len(cw) == 0 or cw.max() == width
+
+
+def test_panel_split_built_in():
+    """Without a call of set_panel_split: tiles of 64 and more, and the FP64 tiles
+    of 48 with blocks of 16 that the default configurations take."""
+    import os
+    import subprocess
+    import sys
+    code = """
+from oracle.elim_list import GREEDY, hqr_elim_list
+from paper_1110_1553_gb300 import hqr
+def split(m, nb, ib, prec):
+    tasks, _, _ = hqr.task_graph(m, 1, nb, ib, hqr_elim_list(m, 1, 2, 1, GREEDY, GREEDY), prec=prec)
+    return bool((tasks[:, 1] > 0).any())
+assert split(2, 48, 16, hqr.FP64) and split(2, 64, 16, hqr.FP64)
+assert not split(1, 48, 16, hqr.FP64) and not split(2, 48, 8, hqr.FP64) and not split(2, 56, 14, hqr.FP64)
+assert not split(2, 48, 16, hqr.FP32) and not split(2, 32, 16, hqr.FP64)
+hqr.set_panel_split(64)
+assert not split(2, 48, 16, hqr.FP64) and split(2, 64, 16, hqr.FP64)
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.run([sys.executable, "-c", code], cwd=root, check=True)
