@@ -1391,9 +1391,19 @@ __device__ __forceinline__ void dot2_merge(double &s1, double &c1, double s2, do
 // binade, and z = fl(s + a x) - s is exact; e = fl(a x - z) then holds what the
 // sum did not take, to 2^(E-106), and goes to c. The sum is (s - sig) + c.
 // Before each group of eight terms, E is raised (s moves to a larger sig, exactly) if
-// a product may exceed 2^(E-5) or s is further than 2^(E-2) from sig: E settles
-// a few binades above the largest product, where Dot2's error follows the
-// running sum's magnitude. Groups whose exponents leave the range take Dot2.
+// a product may exceed 2^(E-5) or s is further than 2^(E-2) from sig. Groups
+// whose exponents leave the range take Dot2.
+//
+// It holds fewer low bits than Dot2. E lies up to 8 binades above the largest
+// product or the sum of magnitudes S = sum |a x| (2^E <= 2^8 S), so n terms of a
+// lane are off by at most n (n + 1) 2^(E-106) <= n (n + 1) 2^-98 S, where Dot2's bound is
+// about n^2 2^-106 S. Against exact rationals, up to 512 terms: both exact for
+// Gaussian FP32 by FP64 products; with products spread over many binades, and
+// FP64 by FP64, 2^-93 to 2^-97 S where Dot2 has 2^-99 to 2^-105. The refinement
+// needs less: the smallest residual it meets is that of a solution rounded to
+// FP64, about 2^-53 S, known to 2^-40 of itself at 2^-93, and R, which turns it
+// into a correction, is FP32. Solutions are as far from the 64-bit ones as with
+// Dot2 (4096 x 4096, kappa 1e6: 1.70e-13, 1.75e-13; 160 uneven: 3.7e-18, 6.5e-18).
 struct BiasedSum {
   double s = 0.0, c = 0.0, sig = 0.0;
   int eb = 0;  // biased exponent of sig (0: none yet)
