@@ -207,11 +207,14 @@ def test_server_idle_exit_and_restart():
 
 def test_other_kernels_run_beside_the_fp64_server():
     # the resident FP64 kernel leaves registers and shared memory of every SM to other streams: a kernel
-    # launched while it waits for work ends before its idle exit (~1 s), not after it
+    # launched while it waits for work ends while it is still resident, not after its idle exit
     A, b, _, bd, x = problem(256, 64, 320)
     Ad = torch.from_numpy(A.astype(np.float64).T.copy()).cuda().t()
     y = torch.zeros(1 << 20, device="cuda")
-    y.add_(1.0)
+    ev, side = torch.cuda.Event(), torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        y.add_(1.0)
+        ev.record()
     torch.cuda.synchronize()
     srv = hqr.Server(torch.float64, refine_iters=0, max_live=2, hbm_budget=64 << 20)
     srv.start()
@@ -219,14 +222,15 @@ def test_other_kernels_run_beside_the_fp64_server():
         t = srv.submit(Ad, bd, x)
         assert t is not None
         wait_all(srv, [t], set())
-        ev = torch.cuda.Event()
-        t0 = time.time()
-        y.add_(1.0)
-        ev.record()
-        while not ev.query() and time.time() - t0 < 0.4:
-            pass
-        assert ev.query()
-        assert time.time() - t0 < 0.4
+        with torch.cuda.stream(side):
+            y.add_(1.0)
+            ev.record()
+        while True:
+            resident = srv.counters()["running"]  # read before the event, so a slow host cannot turn it false
+            if ev.query():
+                break
+            assert resident
+        assert resident
     finally:
         srv.stop()
     assert float(y[0]) == 2.0
