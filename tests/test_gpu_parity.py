@@ -426,6 +426,40 @@ def test_apply_q_block_widths(dtype):
             assert err <= (1e-12 if dtype == "f64" else 5e-6) * np.linalg.norm(B), (k, trans)
 
 
+@pytest.mark.parametrize("prec,nb,ib", [("f64", 64, 16), ("f64", 256, 32), ("f32", 64, 16), ("tensor", 128, 128)])
+def test_reflector_scalars(prec, nb, ib):
+    """beta, tau and v of reflectors of (alpha, x) over the range whose columns are
+    used unscaled, against 60 digits: A = [diag(alpha); diag(x)] killed by one TSQRT
+    has nb independent ones. In units u of rounding (2^-53, FP32 2^-24): n2 =
+    alpha^2 + x^2 carries 2 (x^2 and the sum), so h = sqrt(n2) 1 of them, 0.5 of the
+    rounded n2 y0 and 1 of its own, 2.5, with the series and Newton steps below
+    0.1: beta within 3. |alpha| / h <= 1 adds the 2.5 of 1 / h (FP32: 3, formed from
+    h) and a rounding to tau in [1, 2]: 4 (5). x / (alpha - beta): 2.5 of h, one
+    each of the sum, the reciprocal and the product: 6."""
+    from decimal import Decimal, getcontext
+    getcontext().prec = 60
+    u = Decimal(2) ** (-53 if prec == "f64" else -24)
+    rng = np.random.default_rng(nb)
+    xr, ar = {"f64": (60, 120), "f32": (19, 39), "tensor": (48, 49)}[prec]  # |x| and |alpha| up to (x: and from 1 over) 2^this
+    dt = np.float64 if prec == "f64" else np.float32
+    for trial in range(6):
+        x = (rng.choice([-1, 1], nb) * 2.0 ** rng.uniform(-xr, xr, nb)).astype(dt)
+        al = (rng.choice([-1, 1], nb) * 2.0 ** rng.uniform(-ar, ar, nb)).astype(dt)
+        near = rng.random(nb) < 0.5  # half of them of one size
+        al[near] = (x[near] * rng.uniform(0.01, 100, near.sum()) * rng.choice([-1, 1], near.sum())).astype(dt)
+        al[:2] = 0.0, -0.0
+        A = torch.from_numpy(np.vstack([np.diag(al), np.diag(x)])).cuda()
+        F = hqr.geqrf(A, nb, ib, hqr_elim_list(2, 1, 2, 1, FLAT, FLAT), tensor=prec == "tensor")
+        R, V, T = F.R().cpu().numpy(), F.tiles().cpu().numpy()[nb:2 * nb], F.T().cpu().numpy()[0, 1, 1]
+        for j in range(nb):
+            a, b = Decimal(float(al[j])), Decimal(float(x[j]))
+            h = (a * a + b * b).sqrt()
+            beta = -h if a >= 0 else h
+            for got, ref, tol in ((R[j, j], beta, 3), (T[j, j % ib], 1 + abs(a) / h, 4 if prec == "f64" else 5),
+                                  (V[j, j], b / (a - beta), 6)):
+                assert abs(Decimal(float(got)) - ref) <= tol * u * abs(ref), (trial, j, got, ref)
+
+
 def test_captured_refactor_between_block_widths():
     """A factorization captured in a CUDA graph gives the same bits when replayed
     after right-hand sides of another block width than those before the capture.
