@@ -207,8 +207,9 @@ def test_server_idle_exit_and_restart():
 
 def test_other_kernels_run_beside_the_fp64_server():
     # the resident FP64 kernel leaves registers and shared memory of every SM to other streams: a kernel
-    # launched while it waits for work ends while it is still resident, not after its idle exit
-    A, b, _, bd, x = problem(256, 64, 320)
+    # launched while it works on a request of several milliseconds ends before that request, not when the
+    # kernel's CTAs leave
+    A, b, _, bd, x = problem(16384, 512, 320)
     Ad = torch.from_numpy(A.astype(np.float64).T.copy()).cuda().t()
     y = torch.zeros(1 << 20, device="cuda")
     ev, side = torch.cuda.Event(), torch.cuda.Stream()
@@ -216,21 +217,21 @@ def test_other_kernels_run_beside_the_fp64_server():
         y.add_(1.0)
         ev.record()
     torch.cuda.synchronize()
-    srv = hqr.Server(torch.float64, refine_iters=0, max_live=2, hbm_budget=64 << 20)
+    srv = hqr.Server(torch.float64, refine_iters=0, max_live=2, hbm_budget=1 << 30)
     srv.start()
     try:
         t = srv.submit(Ad, bd, x)
         assert t is not None
-        wait_all(srv, [t], set())
         with torch.cuda.stream(side):
             y.add_(1.0)
             ev.record()
         while True:
-            resident = srv.counters()["running"]  # read before the event, so a slow host cannot turn it false
+            working = srv.progress(t)[0] < srv.progress(t)[1]  # read before the event: a slow host cannot turn it false
             if ev.query():
                 break
-            assert resident
-        assert resident
+            assert working
+        assert working
+        wait_all(srv, [t], set())
     finally:
         srv.stop()
     assert float(y[0]) == 2.0
