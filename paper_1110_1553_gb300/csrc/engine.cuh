@@ -982,6 +982,7 @@ __host__ __device__ inline bool update_resident(int nb, int ib, int w) {
 // W(i,j): every thread takes one unit, in FP32 a 4 x 4 block of W over one of
 // up to 16 parts of the K rows (G parts, in FP64 one element and up to 4 parts);
 // the parts are summed in order through scr. `un` holds the thread's unit.
+// (FP32: at most 8 x 22 blocks, as slabs of a resident tile have fewer than 90 columns.)
 struct TnUnit {
   int mt, g, G;  // output (block), part, parts
   bool on;
@@ -1002,56 +1003,52 @@ __device__ __forceinline__ void resident_tn(const TnUnit &un, float *W, const fl
                                             int ib_, int Nj, const float *Ct, float *scr) {
   const int ib = IB ? IB : ib_, ti = (ib + 3) >> 2, T = ti * ((Nj + 3) >> 2), G = un.G;
   const int Kc = (((K + G - 1) / G) + 3) & ~3;
-  if (T * G <= NT) {
-    if (un.on) {
-      const int i0 = (un.mt % ti) * 4, j0 = (un.mt / ti) * 4;
-      float acc[4][4];
+  if (un.on) {
+    const int i0 = (un.mt % ti) * 4, j0 = (un.mt / ti) * 4;
+    float acc[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+    const int k1 = min(K, (un.g + 1) * Kc);
+    const float *vp[4], *cp[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) vp[a] = V + min(i0 + a, ib - 1) * lds;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) cp[b] = Cm + min(j0 + b, Nj - 1) * lds;
+#pragma unroll 2
+    for (int k = un.g * Kc; k < k1; k += 4) {
+      float4 v4[4], c4[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) v4[a] = *reinterpret_cast<const float4 *>(vp[a] + k);
+#pragma unroll
+      for (int b = 0; b < 4; ++b) c4[b] = *reinterpret_cast<const float4 *>(cp[b] + k);
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-      const int k1 = min(K, (un.g + 1) * Kc);
-      const float *vp[4], *cp[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) vp[a] = V + min(i0 + a, ib - 1) * lds;
-#pragma unroll
-      for (int b = 0; b < 4; ++b) cp[b] = Cm + min(j0 + b, Nj - 1) * lds;
-#pragma unroll 2
-      for (int k = un.g * Kc; k < k1; k += 4) {
-        float4 v4[4], c4[4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) v4[a] = *reinterpret_cast<const float4 *>(vp[a] + k);
-#pragma unroll
-        for (int b = 0; b < 4; ++b) c4[b] = *reinterpret_cast<const float4 *>(cp[b] + k);
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            acc[a][b] = fmaf(v4[a].x, c4[b].x, acc[a][b]);
-            acc[a][b] = fmaf(v4[a].y, c4[b].y, acc[a][b]);
-            acc[a][b] = fmaf(v4[a].z, c4[b].z, acc[a][b]);
-            acc[a][b] = fmaf(v4[a].w, c4[b].w, acc[a][b]);
-          }
-      }
-      // row a of the block at (a T G + unit) * 4: consecutive threads, consecutive 16 bytes
-      float4 *dst = reinterpret_cast<float4 *>(scr) + un.g * T + un.mt;
-#pragma unroll
-      for (int a = 0; a < 4; ++a) dst[a * T * G] = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+        for (int b = 0; b < 4; ++b) {
+          acc[a][b] = fmaf(v4[a].x, c4[b].x, acc[a][b]);
+          acc[a][b] = fmaf(v4[a].y, c4[b].y, acc[a][b]);
+          acc[a][b] = fmaf(v4[a].z, c4[b].z, acc[a][b]);
+          acc[a][b] = fmaf(v4[a].w, c4[b].w, acc[a][b]);
+        }
     }
-    __syncthreads();
-    for (int o = threadIdx.x; o < ib * Nj; o += NT) {
-      const int i = o % ib, j = o / ib;
-      const float *q = scr + ((i & 3) * T * G + (i >> 2) + (j >> 2) * ti) * 4 + (j & 3);
-      float s = Ct ? Ct[i + j * lds] : 0.f;
-      float r = 0.f;
-#pragma unroll 4
-      for (int g = 0; g < G; ++g) r += q[g * T * 4];
-      W[o] = s + r;
-    }
-    __syncthreads();
-  } else {
-    gemm_tn(W, ib, V, lds, Cm, lds, K, ib, Nj, Ct, lds, scr);
+    // row a of the block at (a T G + unit) * 4: consecutive threads, consecutive 16 bytes
+    float4 *dst = reinterpret_cast<float4 *>(scr) + un.g * T + un.mt;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) dst[a * T * G] = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
   }
+  __syncthreads();
+  for (int o = threadIdx.x; o < ib * Nj; o += NT) {
+    const int i = o % ib, j = o / ib;
+    const float *q = scr + ((i & 3) * T * G + (i >> 2) + (j >> 2) * ti) * 4 + (j & 3);
+    float s = Ct ? Ct[i + j * lds] : 0.f;
+    float r = 0.f;
+#pragma unroll 4
+    for (int g = 0; g < G; ++g) r += q[g * T * 4];
+    W[o] = s + r;
+  }
+  __syncthreads();
 }
 
 template <int IB>
