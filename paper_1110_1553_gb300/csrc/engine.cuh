@@ -824,8 +824,9 @@ __device__ __noinline__ void scale_columns(int mode, Real *P, int ld, int L, int
 // FP64 it is bound by the chain of warp 0's instructions (64 cycles each), and
 // for blocks of 32 columns by the FP64 pipe; in FP32 by latencies. Cycles per
 // column (TS, one CTA): 64 x 16 FP64 3200, 256 x 32 FP64 11200, 128 x 16 FP32
-// 1700; block tasks of the whole engine: 64 x 16 FP64 68 -> 29 us, 128 x 32
-// 273 -> 155 us against one CTA-wide reduction after the other.
+// 1700; TSQRT block tasks in a factorization: 64 x 16 FP64 28 us (512^2), 128 x 32
+// 144 us (2000^2), where one CTA-wide reduction after the other took 69 and
+// 273 us, 128 x 16 FP32 16 us.
 template <typename Real>
 __device__ void factor_block(int mode, Real *P, int ld, int L, int ib, Real *Rt, int ldt, int q0, Real *Tq, int ldq,
                              Real *G, Shared<Real> &sh) {
@@ -1496,8 +1497,10 @@ __device__ __forceinline__ double tile_dot(const M *m, int ld, bool transposed, 
 // registers), then the blocks at distance d = 1, 2, ... above them, X_ab = -X_aa
 // S with S = sum over a < l <= b of R_al X_lb kept in X_ab's place in between.
 // Zero diagonal entries are reported to singular(column) and inverted to 0.
-// FP64-pipe bound (n^3 / 6 FMAs: 85 us for 128); one thread per column with its
-// operands from global memory took 970 us.
+// 183 us for a tile of 128; one thread per column with its operands from global
+// memory took 970 us. The n^3 / 6 FMAs are 85 us of an SM's FP64 pipe; beyond
+// them, lanes of the diagonal blocks multiply zeros, and the operands of the
+// blocks above come from L2, one barrier per distance.
 template <typename Real, typename F>
 __device__ void triangle_inverse(const Real *R, double *X, int nb, int n, F singular) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
