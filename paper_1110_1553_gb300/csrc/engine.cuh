@@ -776,9 +776,9 @@ __device__ __noinline__ void flag_column(unsigned key, int c, Shared<Real> &sh) 
 // Looks at the size of column c by the eight lanes of its group: pc[0 .. np) and
 // rc[0 .. nr), its parts in the killed tile (GE: the tile itself) and in R. Every
 // block runs through this once and pays for its instructions more than for
-// its loads: with the shift found here, two loops and the scaling inlined
-// 512^2 FP64 QR + Q took 2.70 ms, so 2.67, without a check 2.65; FP32 2500 x 1700
-// 13.6, 13.45 and 13.4; FP32 with blocks of 8 loses most, 3 to 4 %.
+// its loads: with the shift found here, two loops and the scaling inlined,
+// 512^2 FP64 QR + Q took 1.5 % more than without a check, so 0.2 to 1 %; 2500 x 1700 FP32
+// 1.6 and 0.4 %. FP32 with blocks of 8 columns loses most, 3 to 4 %.
 template <typename Real>
 __device__ __forceinline__ void look_at_column(const Real *pc, int np, const Real *rc, int nr, int c, Shared<Real> &sh) {
   const int lane = threadIdx.x & 31;
