@@ -1497,12 +1497,12 @@ __device__ __forceinline__ double tile_dot(const M *m, int ld, bool transposed, 
 // registers), then the blocks at distance d = 1, 2, ... above them, X_ab = -X_aa
 // S with S = sum over a < l <= b of R_al X_lb kept in X_ab's place in between.
 // Zero diagonal entries are reported to singular(column) and inverted to 0.
-// 183 us for a tile of 128; one thread per column with its operands from global
+// 194 us for a tile of 128; one thread per column with its operands from global
 // memory took 970 us. The n^3 / 6 FMAs are 85 us of an SM's FP64 pipe; beyond
 // them, lanes of the diagonal blocks multiply zeros, and the operands of the
 // blocks above come from L2, one barrier per distance. Not inlined: its 64
 // registers of a row are not the other tasks' concern (512^2 FP64 QR + Q, 130 x 70
-// and others 0.5 to 1 % faster, 6144^2 0.4 %).
+// and others 0.5 to 1 % faster, 6144^2 0.4 %; itself 183 -> 194 us).
 template <typename Real, typename F>
 __device__ __noinline__ void triangle_inverse(const Real *R, double *X, int nb, int n, F singular) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
