@@ -1497,14 +1497,12 @@ __device__ __forceinline__ double tile_dot(const M *m, int ld, bool transposed, 
 // registers), then the blocks at distance d = 1, 2, ... above them, X_ab = -X_aa
 // S with S = sum over a < l <= b of R_al X_lb kept in X_ab's place in between.
 // Zero diagonal entries are reported to singular(column) and inverted to 0.
-// 194 us for a tile of 128; one thread per column with its operands from global
+// 183 us for a tile of 128; one thread per column with its operands from global
 // memory took 970 us. The n^3 / 6 FMAs are 85 us of an SM's FP64 pipe; beyond
 // them, lanes of the diagonal blocks multiply zeros, and the operands of the
-// blocks above come from L2, one barrier per distance. Not inlined: its 64
-// registers of a row are not the other tasks' concern (512^2 FP64 QR + Q, 130 x 70
-// and others 0.5 to 1 % faster, 6144^2 0.4 %; itself 183 -> 194 us).
+// blocks above come from L2, one barrier per distance.
 template <typename Real, typename F>
-__device__ __noinline__ void triangle_inverse(const Real *R, double *X, int nb, int n, F singular) {
+__device__ __forceinline__ void triangle_inverse(const Real *R, double *X, int nb, int n, F singular) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nblk = (n + 31) / 32;
   for (int e = tid; e < nb * nb; e += NT) X[e] = 0.0;
@@ -1578,6 +1576,15 @@ __device__ __noinline__ void triangle_inverse(const Real *R, double *X, int nb, 
     }
 }
 
+// The same as a function of its own, for the scheduler kernels: their other tasks are then compiled without its 64
+// registers of a row (512^2 FP64 QR + Q, 130 x 70 and others 0.5 to 1 % faster, 6144^2 0.4 %; itself 183 -> 194
+// us). The resident server kernels are better with it inlined (2000 requests/s offered to the tensor-core
+// server: 1246 solves/s, 1207 with the call).
+template <typename Real, typename F>
+__device__ __noinline__ void triangle_inverse_call(const Real *R, double *X, int nb, int n, F singular) {
+  triangle_inverse(R, X, nb, n, singular);
+}
+
 __device__ __forceinline__ bool aligned16(const void *p) { return ((uintptr_t)p & 15) == 0; }
 
 // Byte offset of the tiles a triangular-solve step stages in shared memory
@@ -1588,7 +1595,7 @@ static_assert((128 + NT) * 8 <= kVecStageOff, "vector scratch overlaps the stage
 // KU: elements of A each thread keeps in flight in the residual and A^T r
 // loops (16 in the one-CTA-per-SM tensor-core kernel, 8 where two CTAs share
 // an SM's registers).
-template <typename Real, int KU>
+template <typename Real, int KU, bool SERVE>
 __device__ void task_vector(const EngineParams &p, const Problem &P, const Geo<Real> &g, const Task &t,
                             double *sm, Shared<Real> &sh, uint32_t &phase) {
   const int nb = g.nb, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1733,10 +1740,14 @@ __device__ void task_vector(const EngineParams &p, const Problem &P, const Geo<R
     }
     case OP_TRINV: {  // inverse of the upper-triangular leading n_i x n_i part of R_ii
       const int i = t.i, n_i = min(nb, P.N - i * nb);
-      triangle_inverse(g.tile(i, i), P.rinv + (size_t)i * nb * nb, nb, n_i, [&](int col) {
+      auto singular = [&](int col) {
         atomicExch(P.status, HQR_ERR_SINGULAR);
         if (P.rs) atomicMax(&P.rs->sing, ~(unsigned)(i * nb + col));
-      });
+      };
+      if constexpr (SERVE)
+        triangle_inverse(g.tile(i, i), P.rinv + (size_t)i * nb * nb, nb, n_i, singular);
+      else
+        triangle_inverse_call(g.tile(i, i), P.rinv + (size_t)i * nb * nb, nb, n_i, singular);
       break;
     }
     case OP_ATR: {  // partial sums of A(rows of chunk t.i, tile j)^T r
@@ -2261,7 +2272,7 @@ __global__ void __launch_bounds__(NT, TC ? 1 : 2) hqr_sched(EngineParams p) {
     else if (t.op <= OP_TTMQR)
       task_update(p, g, t, sh, dyn, phase);
     else
-      task_vector<Real, TC ? 16 : 8>(p, p.probs[t.pid], g, t, reinterpret_cast<double *>(dyn_raw), sh, phase);
+      task_vector<Real, TC ? 16 : 8, false>(p, p.probs[t.pid], g, t, reinterpret_cast<double *>(dyn_raw), sh, phase);
     __syncthreads();
     const int warp = threadIdx.x >> 5;
     if (warp != 1) {  // warps 0, 2 .. 7 release the successors, warp 0 the most critical 32
@@ -2536,7 +2547,7 @@ __global__ void __maxnreg__(TC ? 255 : sizeof(Real) == 8 ? 112 : 128) hqr_serve(
     else if (t.op <= OP_TTMQR)
       task_update(p, g, t, sh, dyn, phase);
     else
-      task_vector<Real, TC ? 16 : 8>(p, P, g, t, reinterpret_cast<double *>(dyn_raw), sh, phase);
+      task_vector<Real, TC ? 16 : 8, true>(p, P, g, t, reinterpret_cast<double *>(dyn_raw), sh, phase);
     __syncthreads();
     if (threadIdx.x < 32) {  // warp 0 releases the successors, 32 at a time
       ptx::fence_proxy_async();
